@@ -1,0 +1,441 @@
+// Bin sort of a few thousand keys by one CTA in shared memory (keys only).
+//
+// The keys are spread over equal stretches of their range, several times more
+// of them than there are keys, so most bins hold no key or one.  One shared
+// atomic per key counts its bin and gives the key a place in it, a scan of the
+// bins gives each bin its start, every key is written once to its place, and
+// the few bins with two or more keys are sorted by the thread that owns them.
+// Equal keys are identical bit patterns, so the places inside a bin may be
+// given in any order: no match masks, no per-warp counters and no second pass
+// are needed, which the stable radix passes spend most of their shared-memory
+// wavefronts on.
+//
+// Four bins share a 32-bit word: 8-bit counts while the keys are counted,
+// then the first place of the word's first bin (14 bits) and the offsets of
+// the other three (6 bits each), so that a key's place is one read away.  A
+// quarter of the words of 32-bit counters are zeroed, scanned and rewritten,
+// or, seen the other way, four times as many bins cost the same and leave
+// fewer keys to sort inside bins.  1e9 int32 / int64 keys, all groups: 5.3 /
+// 7.3 ms with 10,240 32-bit counters.
+//
+// Where the stretches do not separate the keys (a word of 32 keys or more),
+// block_bin_sort_wide takes over: 32-bit counters, bins of up to 32 *
+// kBinWarpKeys keys sorted by one warp each (bitonic), and if some bin is larger
+// still the merge sort of Algorithm 3, so any input is sorted in bounded time.
+#pragma once
+
+#include "common.cuh"
+#include "smem_sort.cuh"
+
+namespace evosort {
+
+constexpr int kBinMax = 1 << 15;     // most bins
+constexpr int kBinThreadKeys = 31;   // longest bin one thread sorts (2^k - 1)
+constexpr int kBinWide = 12;         // bins per thread of block_bin_sort_wide
+constexpr int kBinWarpKeys = 16;     // keys per lane of the warp sort
+
+// Bytes of the second buffer of n keys: the words of the bins, or the merge
+// sort's other array.
+__host__ __device__ constexpr size_t bin_scratch_bytes(int n, int w, int words) {
+    return (size_t)n * w > (size_t)words * 4 ? (size_t)n * w : (size_t)words * 4;
+}
+
+// Position of d = key - low in [0, 2^32): d shifted so that the widest one
+// (lz leading zeros, of 64 bits) starts at bit 31.
+__device__ __forceinline__ uint32_t norm32(uint32_t d, int lz) { return d << (lz - 32); }
+__device__ __forceinline__ uint32_t norm32(uint64_t d, int lz) {
+    const uint32_t lo = (uint32_t)d, hi = (uint32_t)(d >> 32);
+    return lz < 32 ? __funnelshift_l(lo, hi, lz) : lo << (lz - 32);
+}
+// Smallest d whose position is at least x.
+__device__ __forceinline__ unsigned long long denorm32(uint32_t x, int lz) {
+    if (lz < 32) return (unsigned long long)x << (32 - lz);
+    const int s = lz - 32;
+    return ((unsigned long long)x + ((1ull << s) - 1ull)) >> s;
+}
+// Cuts [0, width] into at most parts equal stretches: part = umulhi(position,
+// mult), below the returned count.  With width < parts every part is one
+// value (part = d).
+__device__ __forceinline__ uint32_t cut_range(unsigned long long width, uint32_t parts, int* lz, uint32_t* mult) {
+    if (width == 0 || parts <= 1u) {
+        *lz = 63;
+        *mult = 0u;
+        return 1u;
+    }
+    const int z = __clzll((long long)width);
+    *lz = z;
+    if (width < (unsigned long long)parts) {   // (parts <= kBinMax, so z >= 49)
+        *mult = 1u << (64 - z);
+        return (uint32_t)width + 1u;
+    }
+    const uint32_t x = norm32((uint64_t)width, z);   // in [2^31, 2^32)
+    *mult = (uint32_t)(((unsigned long long)parts << 32) / ((unsigned long long)x + 1ull));
+    return parts;
+}
+// The same for many cuts of one value each in turn, where a few parts fewer do
+// not matter: one float division instead of a 64-bit one.
+__device__ __forceinline__ void cut_range_near(unsigned long long width, uint32_t parts, int* lz, uint32_t* mult) {
+    if (width == 0) {
+        *lz = 63;
+        *mult = 0u;
+        return;
+    }
+    const int z = __clzll((long long)width);
+    *lz = z;
+    if (width < (unsigned long long)parts) {
+        *mult = 1u << (64 - z);
+        return;
+    }
+    // below the exact quotient by more than the float roundings add up to
+    const float x = (float)norm32((uint64_t)width, z);
+    *mult = (uint32_t)(__fdividef((float)parts * 65536.0f, x) * 65535.9f * 0.999999f);
+}
+// Smallest position of part j >= 1.
+__device__ __forceinline__ uint32_t part_start(uint32_t j, uint32_t mult) {
+    return (uint32_t)((((unsigned long long)j << 32) + mult - 1ull) / mult);
+}
+
+template <typename U, int NT>
+struct BinShared {
+    U mn[NT / 32], mx[NT / 32];
+    uint32_t wsum[NT / 32];
+    uint32_t nlist, big;
+    uint32_t list[512];   // bins left to the warps: first position | length << 16
+};
+
+// Smallest and largest of the CTA's keys (element i * NT + thread < n).
+template <typename U, int NT, int KPT>
+__device__ __forceinline__ void block_extent(const U (&key)[KPT], int n, BinShared<U, NT>& sh, U* lo, U* hi) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    U mn = ~(U)0, mx = 0;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        if (i * NT + tid < n) {
+            mn = key[i] < mn ? key[i] : mn;
+            mx = key[i] > mx ? key[i] : mx;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const U a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+        mn = a < mn ? a : mn;
+        mx = b > mx ? b : mx;
+    }
+    if (lane == 0) {
+        sh.mn[warp] = mn;
+        sh.mx[warp] = mx;
+    }
+    __syncthreads();
+    mn = lane < NW ? sh.mn[lane] : ~(U)0;
+    mx = lane < NW ? sh.mx[lane] : (U)0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const U a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+        mn = a < mn ? a : mn;
+        mx = b > mx ? b : mx;
+    }
+    *lo = mn;
+    *hi = mx;
+}
+
+// Insertion sort of k[0..c) in shared memory by one thread.
+template <typename U>
+__device__ __forceinline__ void bin_insertion(U* k, int c) {
+    const U a = k[0], b = k[1];
+    if (b < a) {
+        k[0] = b;
+        k[1] = a;
+    }
+    for (int i = 2; i < c; ++i) {
+        const U x = k[i];
+        int j = i;
+        while (j > 0) {
+            const U y = k[j - 1];
+            if (!(y > x)) break;
+            k[j] = y;
+            --j;
+        }
+        if (j < i) k[j] = x;
+    }
+}
+
+// Sort of k[0..c), c <= 32 * kBinWarpKeys, by one warp.
+template <typename U>
+__device__ __noinline__ void bin_warp_sort(U* k, int c) {
+    const int lane = threadIdx.x & 31;
+    U x[kBinWarpKeys];
+#pragma unroll
+    for (int r = 0; r < kBinWarpKeys; ++r) {
+        const int i = lane * kBinWarpKeys + r;
+        x[r] = i < c ? k[i] : ~(U)0;
+    }
+    warp_bitonic_sort<U, kBinWarpKeys>(x);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kBinWarpKeys; ++r) {
+        const int i = lane * kBinWarpKeys + r;
+        if (i < c) k[i] = x[r];
+    }
+}
+
+// The keys of k0 stand in their bins (starts in k1, ends of a thread's last
+// bin in run, multi: its bins of two or more keys): sorts the bins, the long
+// ones (heavy: there are some) by a warp each, or everything if some bin is
+// longer still.
+template <typename U, int NT, int BPT>
+__device__ __forceinline__ const U* bin_finish(U* k0, U* k1, int n, uint32_t multi, uint32_t run, bool heavy,
+                                               BinShared<U, NT>& sh) {
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const uint32_t* const own = (const uint32_t*)k1 + tid * BPT;
+    if (tid == 0) sh.nlist = sh.big = 0u;
+    __syncthreads();
+    while (multi) {
+        const int q = __ffs((int)multi) - 1;
+        multi &= multi - 1u;
+        const uint32_t at = own[q], next = q + 1 < BPT ? own[q + 1] : run;
+        const int m = (int)(next - at);
+        if (m <= kBinThreadKeys) {
+            bin_insertion(k0 + at, m);
+        } else if (m <= 32 * kBinWarpKeys) {
+            sh.list[atomicAdd(&sh.nlist, 1u)] = at | (uint32_t)m << 16;   // n / (kBinThreadKeys + 1) entries at most
+        } else {
+            sh.big = 1u;
+        }
+    }
+    __syncthreads();
+    if (!heavy) return k0;
+    if (sh.big) return smem_merge_sort<U, false, 8>(k0, k1, nullptr, nullptr, n, 8) ? k1 : k0;
+    const int m = (int)sh.nlist;
+    for (int e = warp; e < m; e += NT / 32) bin_warp_sort(k0 + (sh.list[e] & 0xFFFFu), (int)(sh.list[e] >> 16));
+    __syncthreads();
+    return k0;
+}
+
+template <int NT, int BPT, typename U>
+__device__ __forceinline__ void bin_zero(U* k1) {
+    uint4* const mine = (uint4*)k1 + threadIdx.x * (BPT / 4);
+#pragma unroll
+    for (int j = 0; j < BPT / 4; ++j) mine[j] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// The same sort with 32-bit counters and any distribution of the keys, which
+// lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per thread.
+template <typename U, int NT, int KPT, int BPT>
+__device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, U* k0, U* k1,
+                                                     BinShared<U, NT>& sh) {
+    static_assert(BPT % 8 == 4 && BPT * NT <= kBinMax, "bins per thread");
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t* const bins = (uint32_t*)k1;
+    // A thread's BPT bins are consecutive and read four at a time; with BPT / 4
+    // odd, a quarter-warp's 16-byte reads fall in different banks.
+    uint4* const mine = (uint4*)bins + tid * (BPT / 4);
+    bin_zero<NT, BPT>(k1);
+    U key[KPT];
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) key[i] = i * NT + tid < n ? k0[i * NT + tid] : (U)0;
+    int lz;
+    uint32_t mult;
+    cut_range(width, (uint32_t)(BPT * NT), &lz, &mult);
+    __syncthreads();
+    if (tid == 0) sh.nlist = sh.big = 0u;
+    // ---- count; the old count is the key's place in its bin
+    uint32_t br[KPT];   // bin | place << 16
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        if (i * NT + tid < n) {
+            // (in range for every key of [lo, lo + width]; never out of the array for any other)
+            const uint32_t b = min(__umulhi(norm32((U)(key[i] - lo), lz), mult), (uint32_t)(BPT * NT - 1));
+            br[i] = b | atomicAdd(&bins[b], 1u) << 16;
+        }
+    }
+    __syncthreads();
+
+    // ---- exclusive scan of the bins
+    uint32_t sum = 0, multi = 0, any = 0;   // multi: bins of two or more keys
+#pragma unroll
+    for (int j = 0; j < BPT / 4; ++j) {
+        const uint4 q = mine[j];
+        sum += q.x + q.y + q.z + q.w;
+        any |= q.x | q.y | q.z | q.w;
+        if (q.x > 1u) multi |= 1u << (4 * j);
+        if (q.y > 1u) multi |= 2u << (4 * j);
+        if (q.z > 1u) multi |= 4u << (4 * j);
+        if (q.w > 1u) multi |= 8u << (4 * j);
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sh.wsum[warp] = inc;
+    __syncthreads();
+    uint32_t run = inc - sum;
+    {
+        uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
+        v = lane < warp ? v : 0u;
+        run += __reduce_add_sync(0xffffffffu, v);
+    }
+#pragma unroll
+    for (int j = 0; j < BPT / 4; ++j) {
+        uint4 q = mine[j];   // read again: registers hold the keys
+        const uint32_t a = run + q.x, b = a + q.y, c = b + q.z, d = c + q.w;
+        q = make_uint4(run, a, b, c);
+        mine[j] = q;
+        run = d;
+    }
+    const bool one_value = width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
+    const bool heavy = __syncthreads_or(!one_value && any > (uint32_t)kBinThreadKeys);
+
+    // ---- every key to its place
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+        if (i * NT + tid < n) k0[bins[br[i] & 0xFFFFu] + (br[i] >> 16)] = key[i];
+    __syncthreads();
+    if (one_value) return k0;
+    return bin_finish<U, NT, BPT>(k0, k1, n, multi, run, heavy, sh);
+}
+
+// Sorts the n keys that the CTA's NT threads hold in registers (key i of a
+// thread is element i * NT + thread; elements from n on are ignored), all in
+// [lo, lo + width].  The words in k1 are zero (bin_zero) and every thread
+// knows it.  WPT words of four bins per thread; (lz, mult) from
+// cut_range(width, 4 * WPT * NT).  k0 holds n keys, k1 bin_scratch_bytes(n, w,
+// WPT * NT) bytes, both 16-byte aligned; n < 2^14.  placed() runs once the
+// registers' keys are in shared memory (the caller may reload them, all of
+// them).  Returns the sorted array (k0 or k1), complete for every thread.
+template <typename U, int NT, int KPT, int WPT, typename F>
+__device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U lo, unsigned long long width, int lz,
+                                                   uint32_t mult, U* k0, U* k1, BinShared<U, NT>& sh,
+                                                   const F& placed) {
+    static_assert(WPT % 8 == 4 && 4 * WPT * NT <= kBinMax && KPT * NT < (1 << 14), "words per thread");
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t* const words = (uint32_t*)k1;
+    // A thread's WPT words are consecutive and read four at a time; with WPT /
+    // 4 odd, a quarter-warp's 16-byte reads fall in different banks.
+    uint4* const mine = (uint4*)words + tid * (WPT / 4);
+
+    // ---- count; the old count is the key's place in its bin
+    uint32_t br[KPT];   // place | bin << 8
+#pragma unroll
+    for (int c = 0; c < KPT; c += 4) {
+        if (c * NT < n) {   // (four columns at a time, so that a short run skips the others)
+#pragma unroll
+            for (int i = c; i < c + 4 && i < KPT; ++i) {
+                if (i * NT + tid < n) {
+                    // (in range for every key of [lo, lo + width]; never out of the array for any other)
+                    const uint32_t b = min(__umulhi(norm32((U)(key[i] - lo), lz), mult), (uint32_t)(4 * WPT * NT - 1));
+                    const uint32_t old = atomicAdd(&words[b >> 2], __funnelshift_l(0u, 1u, 8u * b));   // by 8 (b mod 4)
+                    br[i] = b << 8 | (__funnelshift_r(old, 0u, 8u * b) & 0xFFu);
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- exclusive scan of the bins.  A count that ran over its 8 bits shows
+    // in the total: it takes 256 from its own and gives at most one away.
+    uint32_t sum = 0, any = 0, multi = 0;   // multi: words with a bin of two or more keys
+#pragma unroll
+    for (int j = 0; j < WPT / 4; ++j) {
+        const uint4 q = mine[j];
+        sum = __dp4a(q.x, 0x01010101u, sum);
+        sum = __dp4a(q.y, 0x01010101u, sum);
+        sum = __dp4a(q.z, 0x01010101u, sum);
+        sum = __dp4a(q.w, 0x01010101u, sum);
+        any |= q.x | q.y | q.z | q.w;
+        if (q.x & 0xFEFEFEFEu) multi |= 1u << (4 * j);
+        if (q.y & 0xFEFEFEFEu) multi |= 2u << (4 * j);
+        if (q.z & 0xFEFEFEFEu) multi |= 4u << (4 * j);
+        if (q.w & 0xFEFEFEFEu) multi |= 8u << (4 * j);
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sh.wsum[warp] = inc;
+    // a word's counts must stay below 64 in all: bins below 16
+    const bool heavy = __syncthreads_or((any & 0xF0F0F0F0u) != 0u);
+    uint32_t run = inc - sum;
+    {
+        const uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
+        run += __reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);
+        if (heavy || __reduce_add_sync(0xffffffffu, v) != (uint32_t)n) {   // the same for every thread
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                if (i * NT + tid < n) k0[i * NT + tid] = key[i];
+            __syncthreads();
+            const U* r = block_bin_sort_wide<U, NT, KPT, kBinWide>(n, lo, width, k0, k1, sh);
+            placed();
+            return r;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < WPT / 4; ++j) {
+        uint4 q = mine[j];   // read again: registers hold the keys
+        auto word = [&](uint32_t w) {   // counts -> first place and offsets
+            const uint32_t p = w * 0x01010101u;   // prefix sums of the four counts
+            const uint32_t v = run << 18 | (p & 0x3Fu) | ((p >> 2) & 0xFC0u) | ((p >> 4) & 0x3F000u);
+            run += p >> 24;
+            return v;
+        };
+        q.x = word(q.x);
+        q.y = word(q.y);
+        q.z = word(q.z);
+        q.w = word(q.w);
+        mine[j] = q;
+    }
+    __syncthreads();
+
+    // ---- every key to its place
+#pragma unroll
+    for (int c = 0; c < KPT; c += 4) {
+        if (c * NT < n) {
+#pragma unroll
+            for (int i = c; i < c + 4 && i < KPT; ++i) {
+                if (i * NT + tid < n) {
+                    const uint32_t b = br[i] >> 8, w = words[b >> 2];
+                    const uint32_t before = ((w << 6) >> (6u * (b & 3u))) & 0x3Fu;   // keys of the word's earlier bins
+                    k0[(w >> 18) + before + (br[i] & 0xFFu)] = key[i];
+                }
+            }
+        }
+    }
+    placed();
+    __syncthreads();
+    if (width < (unsigned long long)(4 * WPT * NT)) return k0;   // a bin holds one value
+
+    // ---- words with several keys in a bin: first the pairs, which are most of
+    // them, so that a warp's lanes stay together; then the longer ones
+    const uint32_t* const own = words + tid * WPT;
+    uint32_t more = 0;
+    while (multi) {
+        const int q = __ffs((int)multi) - 1;
+        multi &= multi - 1u;
+        const uint32_t at = own[q] >> 18, next = q + 1 < WPT ? own[q + 1] >> 18 : run;
+        if (next - at == 2u) {
+            const U a = k0[at], b = k0[at + 1];
+            if (b < a) {
+                k0[at] = b;
+                k0[at + 1] = a;
+            }
+        } else {
+            more |= 1u << q;
+        }
+    }
+    while (more) {
+        const int q = __ffs((int)more) - 1;
+        more &= more - 1u;
+        const uint32_t at = own[q] >> 18, next = q + 1 < WPT ? own[q + 1] >> 18 : run;
+        bin_insertion(k0 + at, (int)(next - at));
+    }
+    __syncthreads();
+    return k0;
+}
+
+}  // namespace evosort

@@ -178,6 +178,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return false;
 }
 
+// L2 prefetch of the 16-byte-aligned part of [p, p + bytes) by the TMA
+// engine (no shared memory is written; nothing outside the range is read).
+__device__ __forceinline__ void prefetch_l2_inner(const void* p, size_t bytes) {
+    const uintptr_t a = ((uintptr_t)p + 15) & ~(uintptr_t)15;
+    const uintptr_t e = ((uintptr_t)p + bytes) & ~(uintptr_t)15;
+    if (e > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
+}
+
 // Digit `shift .. shift+d` of a key, with 64-bit keys split into words so the
 // shift is one funnel shift.
 __device__ __forceinline__ uint32_t digit_of(uint32_t k, int shift, uint32_t mask) {

@@ -1,0 +1,450 @@
+// Sort of one long run of keys by one CTA (keys only): segments of a batch
+// that shared memory does not hold, and buckets of the partition sort that
+// came out too large for it.
+//
+//   cta_split_sort   cuts the run's sampled key range into equal parts, moves
+//                    the keys to their parts through the other buffer (one
+//                    read to count, one read and one write to move, unstable:
+//                    one shared atomic per key), then sorts runs of whole
+//                    parts in shared memory (bin_sort.cuh).  A part that is
+//                    still too large is cut once more, over its own range;
+//   cta_radix_sort   the LSD radix passes of Algorithms 4a/4b by one CTA, for
+//                    what two cuts do not separate (many equal keys among
+//                    others).  The CTA walks the tiles in order, so running
+//                    digit offsets replace a look-back.
+#pragma once
+
+#include "bin_sort.cuh"
+#include "common.cuh"
+
+namespace evosort {
+
+constexpr int kCtaThreads = 512;
+constexpr int kCtaWarps = kCtaThreads / 32;
+constexpr int kCtaParts = 1024;      // most parts of one cut
+constexpr int kCtaWords = 12;        // words of four bins per thread of a local sort
+constexpr int kCtaFewWords = 4;      // the same for short runs
+constexpr int kCtaFewKeys = 1536;    // longest run they are used for
+
+// keys per thread of a local sort, and of a tile on its way to the parts
+template <typename U>
+__host__ __device__ constexpr int cta_kpt() { return sizeof(U) == 4 ? 16 : 12; }
+template <typename U>
+__host__ __device__ constexpr int cta_cap() { return kCtaThreads * cta_kpt<U>(); }
+// keys per part aimed at: several parts per local sort
+template <typename U>
+__host__ __device__ constexpr int cta_target() { return sizeof(U) == 4 ? 1536 : 1024; }
+// Dynamic shared memory: two buffers of a local sort (the radix passes use
+// them too), then the ends of the parts of both cuts.
+template <typename U>
+__host__ __device__ constexpr size_t cta_buf_bytes() {
+    return (size_t)cta_cap<U>() * sizeof(U) + bin_scratch_bytes(cta_cap<U>(), (int)sizeof(U), kCtaWords * kCtaThreads);
+}
+template <typename U>
+__host__ __device__ constexpr size_t cta_smem_bytes() { return cta_buf_bytes<U>() + (size_t)kCtaParts * 8; }
+
+template <typename U>
+struct CtaShared {
+    BinShared<U, kCtaThreads> bin;
+    uint32_t scan[kCtaWarps + 1];
+    uint32_t next, end, below, above, longest;
+    int active[sizeof(U)];
+};
+
+// Key maps of the first load and the last store: integers are mapped by one
+// xor (which is its own inverse), floats by the general map.
+template <typename U>
+struct XorMap {
+    U c;
+    __device__ __forceinline__ explicit XorMap(const KeyMap& m) : c((U)(m.s ^ m.x)) {}
+    __device__ __forceinline__ U operator()(U k) const { return k ^ c; }
+};
+template <typename U>
+struct FloatIn {
+    KeyMap m;
+    __device__ __forceinline__ explicit FloatIn(const KeyMap& k) : m(k) {}
+    __device__ __forceinline__ U operator()(U k) const { return map_fwd(k, m); }
+};
+template <typename U>
+struct FloatOut {
+    KeyMap m;
+    __device__ __forceinline__ explicit FloatOut(const KeyMap& k) : m(k) {}
+    __device__ __forceinline__ U operator()(U k) const { return map_inv(k, m); }
+};
+struct AsIs {
+    template <typename U>
+    __device__ __forceinline__ U operator()(U k) const { return k; }
+};
+
+// Local sort of n <= cta_cap() keys held in registers (mapped), in [lo, lo +
+// width]; store(position, key) receives the sorted keys.
+template <typename U, typename S>
+__device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int n, U lo, unsigned long long width,
+                                               unsigned char* smem, CtaShared<U>& sh, const S& store) {
+    U* k0 = (U*)smem;
+    U* k1 = k0 + cta_cap<U>();
+    int lz;
+    uint32_t mult;
+    const U* r;
+    if (n <= kCtaFewKeys) {
+        bin_zero<kCtaThreads, kCtaFewWords>(k1);
+        __syncthreads();
+        cut_range_near(width, (uint32_t)(4 * kCtaFewWords * kCtaThreads), &lz, &mult);
+        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaFewWords>(key, n, lo, width, lz, mult, k0, k1, sh.bin, []() {});
+    } else {
+        bin_zero<kCtaThreads, kCtaWords>(k1);
+        __syncthreads();
+        cut_range_near(width, (uint32_t)(4 * kCtaWords * kCtaThreads), &lz, &mult);
+        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaWords>(key, n, lo, width, lz, mult, k0, k1, sh.bin, []() {});
+    }
+    for (int i = threadIdx.x; i < n; i += kCtaThreads) store(i, r[i]);
+    __syncthreads();
+}
+
+// LSD radix sort of the len mapped keys in a (other buffer b); the sorted
+// keys, through out(), end in fin (a or b).  8-bit digits; digits that are
+// equal in all keys are skipped.
+template <typename U, typename M>
+__device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, uint32_t len, M out, unsigned char* smem,
+                                            CtaShared<U>& sh) {
+    constexpr int NP = sizeof(U);
+    constexpr int BINS = 256;
+    constexpr int KPT = 8;
+    constexpr uint32_t TILE = kCtaThreads * KPT;
+    uint32_t* s_hist = (uint32_t*)smem;                 // NP * BINS
+    uint32_t* s_run = s_hist + NP * BINS;               // BINS running offsets
+    uint32_t* s_excl = s_run + BINS;                    // BINS tile offsets
+    uint32_t* s_tcnt = s_excl + BINS;                   // BINS tile counts
+    uint32_t* s_match = s_tcnt + BINS;                  // warps * BINS match masks
+    uint16_t* s_whist = (uint16_t*)(s_match + kCtaWarps * BINS);   // warps * BINS
+    U* s_r = (U*)(s_whist + kCtaWarps * BINS);          // TILE keys
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < NP * BINS; i += kCtaThreads) s_hist[i] = 0;
+    if (tid < NP) sh.active[tid] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (uint32_t i = tid; i < len; i += kCtaThreads) {
+        const U k = a[i];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) atomicAdd(&s_hist[p * BINS + digit_of(k, 8 * p, 0xFFu)], 1u);
+    }
+    __syncthreads();
+    for (int i = tid; i < NP * BINS; i += kCtaThreads)
+        if (s_hist[i] != 0 && s_hist[i] != len) sh.active[i / BINS] = 1;
+    __syncthreads();
+    int nact = 0;
+    for (int p = 0; p < NP; ++p) nact += sh.active[p];
+    U* src = a;
+    U* dst = b;
+    const uint32_t lt = lanemask_lt();
+    for (int p = 0; p < NP; ++p) {
+        if (!sh.active[p]) continue;
+        const int shift = 8 * p;
+        {
+            const uint32_t c = tid < BINS ? s_hist[p * BINS + tid] : 0u;
+            uint32_t tot;
+            const uint32_t ex = block_exclusive_scan<kCtaThreads>(c, sh.scan, &tot);
+            if (tid < BINS) s_run[tid] = ex;
+        }
+        __syncthreads();
+        for (uint32_t t0 = 0; t0 < len; t0 += TILE) {
+            const int valid = len - t0 < TILE ? (int)(len - t0) : (int)TILE;
+            uint16_t* wh = s_whist + warp * BINS;
+            uint32_t* wm = s_match + warp * BINS;
+            for (int i = lane; i < BINS; i += 32) {
+                wm[i] = 0u;
+                if ((i & 1) == 0) ((uint32_t*)wh)[i >> 1] = 0u;
+            }
+            __syncwarp();
+            U key[KPT];
+            uint32_t dr[KPT];
+            const int wofs = warp * 32 * KPT + lane;
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const int s = wofs + 32 * i;
+                key[i] = s < valid ? src[t0 + s] : ~(U)0;
+            }
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const uint32_t dig = digit_of(key[i], shift, 0xFFu);
+                atomicOr(&wm[dig], 1u << lane);
+                __syncwarp();
+                const uint32_t peers = wm[dig];
+                __syncwarp();
+                const int leader = 31 - __clz(peers);
+                uint32_t old = 0;
+                if (lane == leader) {
+                    old = wh[dig];
+                    wh[dig] = (uint16_t)(old + __popc(peers));
+                    wm[dig] = 0u;
+                }
+                old = __shfl_sync(0xffffffffu, old, leader);
+                dr[i] = dig | ((old + __popc(peers & lt)) << 16);
+                __syncwarp();
+            }
+            __syncthreads();
+            uint32_t tc = 0;
+            if (tid < BINS) {
+                for (int w = 0; w < kCtaWarps; ++w) {
+                    const uint32_t c = s_whist[w * BINS + tid];
+                    s_whist[w * BINS + tid] = (uint16_t)tc;
+                    tc += c;
+                }
+                s_tcnt[tid] = tc;
+            }
+            {
+                uint32_t tot;
+                const uint32_t ex = block_exclusive_scan<kCtaThreads>(tc, sh.scan, &tot);
+                if (tid < BINS) s_excl[tid] = ex;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                if (wofs + 32 * i < valid) {
+                    const uint32_t dig = dr[i] & 0xFFFFu;
+                    s_r[s_excl[dig] + wh[dig] + (dr[i] >> 16)] = key[i];
+                }
+            }
+            __syncthreads();
+            for (int s = tid; s < valid; s += kCtaThreads) {
+                const U k = s_r[s];
+                const uint32_t dig = digit_of(k, shift, 0xFFu);
+                dst[s_run[dig] + (s - s_excl[dig])] = k;
+            }
+            __syncthreads();
+            if (tid < BINS) s_run[tid] += s_tcnt[tid];
+            __syncthreads();
+        }
+        U* t = src;
+        src = dst;
+        dst = t;
+    }
+    for (uint32_t i = tid; i < len; i += kCtaThreads) fin[i] = out(src[i]);
+    __syncthreads();
+}
+
+// Sort of the len keys of src: in() maps a key on its load, out() on its last
+// store.  The parts are laid out in part (as long as src); the sorted keys end
+// in fin, which is src or part.  LEVEL 0 cuts too large parts again.
+template <typename U, int LEVEL, typename MI, typename MO>
+__device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
+                                               unsigned char* smem, CtaShared<U>& sh);
+template <typename U, typename MO>
+__device__ __noinline__ void cta_split_again(U* src, U* part, U* fin, uint32_t len, MO out, unsigned char* smem,
+                                             CtaShared<U>& sh) {
+    cta_split_impl<U, 1>(src, part, fin, len, AsIs(), out, smem, sh);
+}
+template <typename U, typename MI, typename MO>
+__device__ __forceinline__ void cta_split_sort(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
+                                               unsigned char* smem, CtaShared<U>& sh) {
+    cta_split_impl<U, 0>(src, part, fin, len, in, out, smem, sh);
+}
+
+template <typename U, int LEVEL, typename MI, typename MO>
+__device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
+                                               unsigned char* smem, CtaShared<U>& sh) {
+    constexpr int KPT = cta_kpt<U>();
+    constexpr int CAP = cta_cap<U>();
+    constexpr uint32_t TILE = CAP;
+    U* s_key = (U*)smem;                                                  // tile buffer, or a local sort's first
+    uint32_t* s_cnt = (uint32_t*)(smem + (size_t)CAP * sizeof(U));        // tile counts (the second buffer)
+    uint32_t* s_at = s_cnt + kCtaParts;
+    uint32_t* s_to = s_at + kCtaParts;
+    // next free place of a part, at last its end
+    uint32_t* s_cur = (uint32_t*)(smem + cta_buf_bytes<U>()) + LEVEL * kCtaParts;
+    const int tid = threadIdx.x, lane = tid & 31;
+
+    // ---- range of the keys, from a sample
+    U lo, hi;
+    {
+        U k[8];
+        const uint32_t stride = len / (8 * kCtaThreads);
+        const int m = stride ? 8 * kCtaThreads : (int)len;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i * kCtaThreads + tid < m) k[i] = in(src[(uint32_t)(i * kCtaThreads + tid) * (stride ? stride : 1u)]);
+        block_extent<U, kCtaThreads, 8>(k, m, sh.bin, &lo, &hi);
+    }
+    const unsigned long long width = (unsigned long long)(U)(hi - lo);
+    if (width == 0) {   // one value, as far as the sample shows
+        bool other = false;
+        for (uint32_t i = tid; i < len; i += kCtaThreads) other |= in(src[i]) != lo;
+        if (!__syncthreads_or(other)) {
+            const U k = out(lo);
+            for (uint32_t i = tid; i < len; i += kCtaThreads) fin[i] = k;
+            __syncthreads();
+            return;
+        }
+    }
+    uint32_t want = (len + (uint32_t)cta_target<U>() - 1u) / (uint32_t)cta_target<U>();
+    if (want > (uint32_t)kCtaParts) want = (uint32_t)kCtaParts;
+    int lz;
+    uint32_t mult;
+    const uint32_t np = cut_range(width, want, &lz, &mult);
+    const bool one_value = width < (unsigned long long)np;
+    // keys outside the sampled range go to the first and the last part
+    auto part_of = [&](U k) {
+        const U d = (k > lo ? k : lo) - lo;
+        return __umulhi(norm32(d < (U)width ? d : (U)width, lz), mult);
+    };
+
+    // ---- count
+    for (int i = tid; i < kCtaParts; i += kCtaThreads) s_cnt[i] = 0u;
+    if (tid == 0) sh.below = sh.above = sh.longest = 0u;
+    __syncthreads();
+    {
+        bool below = false, above = false;
+        auto one = [&](U raw) {
+            const U k = in(raw);
+            below |= k < lo;
+            above |= k > hi;
+            atomicAdd(&s_cnt[part_of(k)], 1u);
+        };
+        uint32_t i = tid;
+        for (; i + 7u * kCtaThreads < len; i += 8u * kCtaThreads) {
+            U k[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) k[u] = src[i + (uint32_t)(u * kCtaThreads)];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) one(k[u]);
+        }
+        for (; i < len; i += kCtaThreads) one(src[i]);
+        if (below) sh.below = 1u;
+        if (above) sh.above = 1u;
+    }
+    __syncthreads();
+    {
+        uint32_t c[2], sum = 0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            c[j] = s_cnt[tid * 2 + j];
+            s_cnt[tid * 2 + j] = 0u;
+            sum += c[j];
+        }
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_scan<kCtaThreads>(sum, sh.scan, &tot);
+        s_cur[tid * 2] = ex;
+        s_cur[tid * 2 + 1] = ex + c[0];
+        atomicMax(&sh.longest, max(c[0], c[1]));
+    }
+    __syncthreads();
+    const bool low_end = sh.below != 0u, high_end = sh.above != 0u;
+    // most keys in one part: not separated by its range
+    if (!one_value && sh.longest > (uint32_t)CAP && sh.longest > len / 2u) {
+        for (uint32_t i = tid; i < len; i += kCtaThreads) src[i] = in(src[i]);
+        __syncthreads();
+        cta_radix_sort<U>(src, part, fin, len, out, smem, sh);
+        return;
+    }
+
+    // ---- move the keys to their parts, a tile at a time
+    {
+        U key[KPT];
+        auto load = [&](uint32_t t0) {
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const uint32_t j = t0 + (uint32_t)(i * kCtaThreads + tid);
+                key[i] = j < len ? src[j] : (U)0;
+            }
+        };
+        load(0);
+        for (uint32_t t0 = 0; t0 < len; t0 += TILE) {
+            const uint32_t valid = min(len - t0, TILE);
+            uint32_t rk[(KPT + 1) / 2];
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                if ((uint32_t)(i * kCtaThreads + tid) < valid) {
+                    key[i] = in(key[i]);
+                    const uint32_t r = atomicAdd(&s_cnt[part_of(key[i])], 1u);
+                    rk[i / 2] = i & 1 ? __byte_perm(rk[i / 2], r, 0x5410) : r;
+                }
+            }
+            __syncthreads();
+            const uint32_t c0 = s_cnt[tid * 2], c1 = s_cnt[tid * 2 + 1];
+            s_cnt[tid * 2] = 0u;
+            s_cnt[tid * 2 + 1] = 0u;
+            uint32_t tot;
+            const uint32_t ex = block_exclusive_scan<kCtaThreads>(c0 + c1, sh.scan, &tot);
+            const uint32_t g0 = s_cur[tid * 2], g1 = s_cur[tid * 2 + 1];
+            s_at[tid * 2] = ex;
+            s_at[tid * 2 + 1] = ex + c0;
+            s_to[tid * 2] = g0 - ex;
+            s_to[tid * 2 + 1] = g1 - (ex + c0);
+            s_cur[tid * 2] = g0 + c0;
+            s_cur[tid * 2 + 1] = g1 + c1;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                if ((uint32_t)(i * kCtaThreads + tid) < valid)
+                    s_key[s_at[part_of(key[i])] + (i & 1 ? rk[i / 2] >> 16 : rk[i / 2] & 0xFFFFu)] = key[i];
+            if (t0 + TILE < len) load(t0 + TILE);
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                const uint32_t s = (uint32_t)(i * kCtaThreads + tid);
+                if (s < valid) {
+                    const U k = s_key[s];
+                    part[s_to[part_of(k)] + s] = k;
+                }
+            }
+            // (the next tile writes s_key, s_at and s_to only after two barriers)
+        }
+        __syncthreads();
+    }
+
+    // ---- runs of whole parts that fit, sorted in shared memory
+    uint32_t f = 0, s = 0;
+    while (f < np) {
+        if (tid < 32) {
+            uint32_t g = f, e = s;
+            for (;;) {
+                const uint32_t i = g + (uint32_t)lane;
+                const uint32_t x = i < np ? s_cur[i] : 0u;
+                const uint32_t m = __ballot_sync(0xffffffffu, i < np && x - s <= (uint32_t)CAP);
+                const int k = m == 0xffffffffu ? 32 : __ffs((int)~m) - 1;
+                if (k > 0) e = __shfl_sync(0xffffffffu, x, k - 1);
+                g += (uint32_t)k;
+                if (k < 32) break;
+            }
+            if (g == f) {   // one part too large
+                e = s_cur[f];
+                g = f + 1u;
+            }
+            if (lane == 0) {
+                sh.next = g;
+                sh.end = e;
+                if (e < len) prefetch_l2_inner(part + e, (size_t)min(len - e, (uint32_t)CAP) * sizeof(U));
+            }
+        }
+        __syncthreads();
+        const uint32_t g = sh.next, e = sh.end, n = e - s;
+        if (n > (uint32_t)CAP) {
+            U* const other = (fin == part ? src : fin) + s;
+            if (one_value && !(f == 0u && low_end) && !(f + 1u == np && high_end)) {
+                for (uint32_t i = s + tid; i < e; i += kCtaThreads) fin[i] = out(part[i]);
+                __syncthreads();
+            } else if (LEVEL == 0) {
+                __syncthreads();   // (sh is used again)
+                cta_split_again<U>(part + s, other, fin + s, n, out, smem, sh);
+            } else {
+                __syncthreads();
+                cta_radix_sort<U>(part + s, other, fin + s, n, out, smem, sh);
+            }
+        } else if (n > 0) {
+            U key[KPT];
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                key[i] = (uint32_t)(i * kCtaThreads + tid) < n ? part[s + (uint32_t)(i * kCtaThreads + tid)] : (U)0;
+            U a, b;
+            block_extent<U, kCtaThreads, KPT>(key, (int)n, sh.bin, &a, &b);
+            cta_local_sort<U>(key, (int)n, a, (unsigned long long)(U)(b - a), smem, sh,
+                              [&](int i, U k) { fin[s + (uint32_t)i] = out(k); });
+        } else {
+            __syncthreads();
+        }
+        f = g;
+        s = e;
+    }
+}
+
+}  // namespace evosort

@@ -1,0 +1,71 @@
+"""GPU parity of the one-CTA sorts of the batched segmented sort (the bin sort
+of a short run, the cuts of a long one and the radix passes behind them)
+against the oracle: lengths at the edges of each, keys that their range
+separates well, badly or not at all."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def evo():
+    import paper_2505_18681_gb300 as evo
+    evo.library()
+    evo.table_clear()
+    return evo
+
+
+def host(t):
+    if t.dtype in (torch.uint32, torch.uint64):
+        s = t.view(torch.int32 if t.dtype == torch.uint32 else torch.int64).cpu().numpy()
+        return s.view(np.uint32 if t.dtype == torch.uint32 else np.uint64)
+    return t.cpu().numpy()
+
+
+def bits(t):
+    a = host(t) if isinstance(t, torch.Tensor) else t
+    return a.view(np.uint32 if a.dtype.itemsize == 4 else np.uint64)
+
+
+def powers(n, seed):
+    """Magnitudes spread over every binary order."""
+    from paper_2505_18681_gb300 import inputs
+    x = inputs.generate("uniform", n, torch.int64, seed=seed, device="cuda")
+    m = (inputs.generate("uniform", n, torch.int64, seed=seed + 1, device="cuda") & 63).clamp(max=62)
+    return (x & ((1 << 62) - 1)) >> m
+
+
+@pytest.mark.parametrize("dtype", [torch.int32, torch.int64, torch.float64], ids=str)
+@pytest.mark.parametrize("kind", ["uniform", "equal", "few", "sparse", "powers", "clusters", "ramp"])
+def test_segments_of_every_shape(evo, dtype, kind):
+    """Segments at the edges of the one-CTA sorts (a short run, a full local
+    sort, one key more, several cuts) whose keys their range separates well,
+    badly or not at all."""
+    lengths = torch.tensor([2, 31, 255, 256, 257, 1535, 1536, 1537, 4096, 4097, 6143, 6144, 6145, 8191, 8192, 8193,
+                            12289, 65536, 100_003, 700_001], dtype=torch.int64)
+    offs = torch.zeros(lengths.numel() + 1, dtype=torch.int64)
+    offs[1:] = torch.cumsum(lengths, 0)
+    n = int(offs[-1])
+    from paper_2505_18681_gb300 import inputs
+    x = inputs.generate("uniform", n, torch.int64, seed=5, device="cuda")
+    if kind == "equal":
+        x = torch.full_like(x, -9)
+    elif kind == "few":
+        x = x % 7
+    elif kind == "sparse":
+        x = torch.where(x % 10 == 0, x >> 33, torch.zeros_like(x))
+    elif kind == "powers":
+        x = powers(n, 6)
+    elif kind == "clusters":    # half of the keys in 300 values far from the rest
+        x = torch.where(x % 2 == 0, (x >> 8) % 300, x)
+    elif kind == "ramp":
+        x = torch.arange(n, dtype=torch.int64, device="cuda") * 5 - n
+    k = x.to(dtype) if dtype != torch.int32 else (x >> (32 if kind in ("uniform", "powers", "clusters") else 0)).to(dtype)
+    want = oracle.segmented_sort(host(k), offs.numpy().astype(np.uint64))
+    evo.segmented_sort(k, offs.cuda())
+    evo.sync()
+    assert np.array_equal(bits(k), bits(want))
