@@ -90,6 +90,7 @@ static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 struct ProfRecord {
     int kind, pass, call;
     int rank;   // adaptive ranking: the variant this launch runs (0: not adaptive)
+    bool same;  // the launch of the record before, its other variant (no events of its own)
     double bytes;
     uint64_t items;
     cudaEvent_t e0, e1;
@@ -139,16 +140,17 @@ void prof_call_end(int call, cudaStream_t s, const PassDesc* dev_desc) {
     }
 }
 
-ProfScope::ProfScope(int call, int kind, int pass, double bytes, uint64_t items, cudaStream_t s, int rank)
+ProfScope::ProfScope(int call, int kind, int pass, double bytes, uint64_t items, cudaStream_t s, int rank, int other)
     : call_(call), idx_(-1), s_(s) {
     if (!g_prof_on || call < 0) return;
-    ProfRecord r{kind, pass, call, rank, bytes, items, nullptr, nullptr};
+    ProfRecord r{kind, pass, call, rank, false, bytes, items, nullptr, nullptr};
     cudaEventCreate(&r.e0);
     cudaEventCreate(&r.e1);
     cudaEventRecord(r.e0, s);
     std::lock_guard<std::mutex> lk(g_prof_mu);
     g_prof.push_back(r);
     idx_ = (int)g_prof.size() - 1;
+    if (other) g_prof.push_back(ProfRecord{kind, pass, call, other, true, bytes, items, nullptr, nullptr});
 }
 
 ProfScope::~ProfScope() {
@@ -229,7 +231,7 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     a.d = pl.digit_bits;
     a.npass = L.npass;
     a.lb64 = L.lb64;
-    // adaptive ranking pays one extra (empty) launch per pass; below a few
+    // adaptive ranking needs the digit counts of many keys to say much; below a few
     // million keys the match-mask ranking alone runs
     const bool adapt = pl.rank_mode == 4 && n >= kAdaptMinKeys;
     const int rank = pl.rank_mode == 4 ? 3 : pl.rank_mode;
@@ -249,6 +251,7 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     const int inplace = (in == out) ? 1 : 0;
 
     cudaError_t e = cudaMemsetAsync(base, 0, L.zero_end, s);
+    const int call = prof_call_begin(a.desc, L.npass + 1, s);
     const int sms = sm_count();
     const size_t hist_smem = (size_t)L.npass * ((size_t)1 << pl.digit_bits) * sizeof(uint32_t);
     size_t hist_grid = (n + 1024 * 16 - 1) / (1024 * 16);
@@ -256,7 +259,6 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     if (hist_grid < 1) hist_grid = 1;
     const int vb = pairs ? 4 : 0;
     const double pass_bytes = 2.0 * (double)n * (w + vb);
-    const int call = prof_call_begin(a.desc, L.npass + 1, s);
     {
         ProfScope ps(call, EVOSORT_K_RADIX_HISTOGRAM, -1, (double)n * w, n, s);
         if (e == cudaSuccess) e = launch_radix_aux(w, 0, hist_grid, hist_smem, s, a, inplace);
@@ -281,9 +283,13 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     }
     const bool reg = pl.pass_kernel == 2;
     for (int p = 0; p < L.npass && e == cudaSuccess; ++p) {
-        for (int v = 0; v < (adapt ? 2 : 1) && e == cudaSuccess; ++v) {
-            const int r = v == 0 ? rank : 1;
-            ProfScope ps(call, EVOSORT_K_RADIX_ONESWEEP, p, pass_bytes, n, s, adapt ? r : 0);
+        // adaptive ranking: the register tile takes both variants in one launch
+        // (a record of each, of which the one that ran is active), the staged
+        // tile has a kernel for each
+        for (int v = 0; v < (adapt && !reg ? 2 : 1) && e == cudaSuccess; ++v) {
+            const int r = adapt && reg ? 4 : (v == 0 ? rank : 1);
+            ProfScope ps(call, EVOSORT_K_RADIX_ONESWEEP, p, pass_bytes, n, s, adapt ? (v == 0 ? rank : 1) : 0,
+                         adapt && reg ? 1 : 0);
             if (reg && w == 4)
                 e = launch_onesweep_reg_u32(pairs, pl.block_size, pl.keys_per_thread, r, L.ntiles, sms, s, a, p);
             else if (reg)
@@ -302,7 +308,7 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     }
     prof_call_end(call, s, a.desc);
     count_launches(3 + (pl.digit_bits == 8 ? 1 : 0) + (pl.digit_bits == 8 && !pairs ? 2 : 0) +
-                   (adapt ? 2 : 1) * L.npass);
+                   (adapt && !reg ? 2 : 1) * L.npass);
     if (e != cudaSuccess) {
         *err = std::string("radix launch: ") + cudaGetErrorString(e);
         return EVOSORT_ERR_CUDA;
@@ -868,17 +874,26 @@ evosort_status evosort_profile(int enable) {
 size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
     std::lock_guard<std::mutex> lk(g_prof_mu);
     size_t k = 0;
+    float launch_ms = 0.f;   // of the last record with events
     for (size_t i = 0; i < g_prof.size(); ++i) {
         ProfRecord& r = g_prof[i];
-        cudaEventSynchronize(r.e1);
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, r.e0, r.e1);
+        if (!r.same) {
+            cudaEventSynchronize(r.e1);
+            launch_ms = 0.f;
+            cudaEventElapsedTime(&launch_ms, r.e0, r.e1);
+        }
+        float ms = launch_ms;
         int active = 1;
         const ProfCall& c = g_prof_calls[r.call];
         if (c.copied) cudaEventSynchronize(c.copied);
         if (c.host_desc) {
-            if (r.kind == EVOSORT_K_RADIX_ONESWEEP && r.pass >= 0 && r.pass < c.ndesc)
+            if (r.kind == EVOSORT_K_RADIX_ONESWEEP && r.pass >= 0 && r.pass < c.ndesc) {
                 active = c.host_desc[r.pass].active && (r.rank == 0 || c.host_desc[r.pass].rank == r.rank);
+                // one launch for both variants: its time goes to the one that
+                // ran (to the first if the pass was skipped)
+                const bool both = r.same || (i + 1 < g_prof.size() && g_prof[i + 1].same);
+                if (both && !active && (r.same || c.host_desc[r.pass].active)) ms = 0.f;
+            }
             if (r.kind == EVOSORT_K_RADIX_FIXUP && r.pass >= 0 && r.pass < c.ndesc)
                 active = c.host_desc[r.pass].fixup != FIX_NONE;
         }
@@ -892,6 +907,7 @@ size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
             out[k].rank = r.rank;
         }
         ++k;
+        if (r.same) continue;
         cudaEventDestroy(r.e0);
         cudaEventDestroy(r.e1);
     }

@@ -93,7 +93,8 @@ void prof_call_end(int call, cudaStream_t s, const PassDesc* dev_desc);
 // Records a CUDA event pair around one launch while instrumentation is on.
 class ProfScope {
   public:
-    ProfScope(int call, int kind, int pass, double bytes, uint64_t items, cudaStream_t s, int rank = 0);
+    // other: a second record of the same launch, for the ranking variant `other`
+    ProfScope(int call, int kind, int pass, double bytes, uint64_t items, cudaStream_t s, int rank = 0, int other = 0);
     ~ProfScope();
   private:
     int call_, idx_;

@@ -100,6 +100,33 @@ __device__ __forceinline__ uint64_t map_inv(uint64_t t, const KeyMap& m) {
 }
 
 // ---------------------------------------------------------------------------
+// Chains of kernels (programmatic dependent launch).  A kernel launched with
+// launch_chain may be set up, and its CTAs placed, while the kernel before it
+// still runs; chain_wait, which every such kernel calls before anything else,
+// holds it until that kernel has ended and its writes are visible.  A kernel
+// that finds nothing to do then costs about 1 us of its stream's time, not 3
+// to 4, and one that works starts without the gap.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_chain(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Relaxed GPU-scope loads/stores for the decoupled look-back slots.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {

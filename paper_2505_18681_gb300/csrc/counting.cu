@@ -42,6 +42,7 @@ __device__ __forceinline__ bool counting_applies(const RadixArgs& a, U* base) {
 
 template <typename U>
 __global__ void __launch_bounds__(kCountThreads) radix_count_values(RadixArgs a, unsigned long long* bins) {
+    chain_wait();
     __shared__ uint32_t s_h[kCountBins];
     U base;
     if (!counting_applies<U>(a, &base)) return;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(kCountThreads) radix_count_values(RadixArgs a,
 
 template <typename U>
 __global__ void __launch_bounds__(kCountThreads) radix_count_fill(RadixArgs a, const unsigned long long* bins) {
+    chain_wait();
     extern __shared__ unsigned long long s_start[];   // kCountBins + 1
     __shared__ unsigned long long s_part[kCountThreads / 32];
     U base;
@@ -183,11 +185,9 @@ cudaError_t launch_counting(const RadixArgs& a, unsigned long long* bins, cudaSt
     const int sms = sm_count();
     const size_t want = (a.n / (16 / sizeof(U)) + kCountThreads - 1) / kCountThreads;
     const unsigned grid = (unsigned)(want < (size_t)sms * 2 ? (want ? want : 1) : (size_t)sms * 2);
-    radix_count_values<U><<<grid, kCountThreads, 0, s>>>(a, bins);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chain(radix_count_values<U>, grid, kCountThreads, 0, s, a, bins);
     if (e != cudaSuccess) return e;
-    radix_count_fill<U><<<grid, kCountThreads, smem, s>>>(a, bins);
-    return cudaGetLastError();
+    return launch_chain(radix_count_fill<U>, grid, kCountThreads, smem, s, a, bins);
 }
 
 }  // namespace

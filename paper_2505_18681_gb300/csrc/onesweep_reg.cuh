@@ -34,6 +34,8 @@
 // per pass against 4.85 ms for the staged kernel at its best tile.
 #pragma once
 
+#include <type_traits>
+
 #include "radix.cuh"
 
 namespace evosort {
@@ -70,13 +72,17 @@ __host__ __device__ constexpr bool reg_shape_ok(int block, int d) { return block
 template <typename U, bool PAIRS, int BLOCK, int KPT, int D, int RANK>
 __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 1024 / BLOCK))
     radix_onesweep_reg(RadixArgs a, int pass) {
+    chain_wait();
     constexpr int WARPS = BLOCK / 32;
     constexpr int TILE = BLOCK * KPT;
     constexpr int bins = 1 << D;
     static_assert(reg_shape_ok(BLOCK, D), "register tile needs BLOCK >= 2 * bins");
     static_assert(RANK != 2, "ranking");
     const PassDesc desc = a.desc[pass];
-    if (!desc.active || (a.adapt && desc.rank != RANK)) return;
+    if (!desc.active) return;
+    // RANK 4: this pass's variant, the same for every thread.  (Two launches of
+    // which one returned cost 2 to 3 us more per pass.)
+    const bool match_any = RANK == 1 || (RANK == 4 && desc.rank == 1);
 
     const int shift = pass * D;
     constexpr uint32_t mask = (uint32_t)(bins - 1);
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 1024 / BLOCK))
     uint32_t* s_rv = (uint32_t*)(smem + (size_t)TILE * sizeof(U));
     uint32_t* s_wc = (uint32_t*)(smem + (size_t)TILE * (sizeof(U) + (PAIRS ? 4 : 0)));
     uint32_t* s_wm = s_wc + WARPS * bins;                                  // rank mode 3 only
-    uint32_t* s_excl = s_wm + (RANK == 3 ? WARPS * bins : 0);              // tile offset of each digit
+    uint32_t* s_excl = s_wm + (RANK != 1 ? WARPS * bins : 0);              // tile offset of each digit
     uint32_t* s_cnt = s_excl + bins;                                       // tile count of each digit
     unsigned long long* s_gbase = (unsigned long long*)(s_cnt + bins);     // global start - tile offset
     uint32_t* s_gbase32 = (uint32_t*)(s_gbase + bins);
@@ -119,7 +125,7 @@ __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 1024 / BLOCK))
     };
     if (tid == 0) claim(0);
     // match masks start at zero; each column's leader clears the words it used
-    if (RANK == 3)
+    if (!match_any)
         for (int i = tid; i < WARPS * bins; i += BLOCK) s_wm[i] = 0u;
     __syncthreads();
 
@@ -169,28 +175,34 @@ __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 1024 / BLOCK))
         // ---- stable rank among equal digits of the warp: columns in input
         // order, lanes in order inside a column
         const uint32_t lt = lanemask_lt();
+        auto rank_columns = [&](auto any) {
 #pragma unroll
-        for (int i = 0; i < KPT; ++i) {
-            const uint32_t d0 = digit_of(key[i], shift, mask);
-            uint32_t p0;
-            if (RANK == 1) {
-                p0 = __match_any_sync(0xffffffffu, d0);
-            } else {
-                atomicOr(&wm[d0], 1u << lane);
-                __syncwarp();
-                p0 = wm[d0];
+            for (int i = 0; i < KPT; ++i) {
+                const uint32_t d0 = digit_of(key[i], shift, mask);
+                uint32_t p0;
+                if (any.value) {
+                    p0 = __match_any_sync(0xffffffffu, d0);
+                } else {
+                    atomicOr(&wm[d0], 1u << lane);
+                    __syncwarp();
+                    p0 = wm[d0];
+                    __syncwarp();
+                }
+                const int l0 = 31 - __clz(p0);
+                uint32_t o0 = 0;
+                if (lane == l0) {
+                    o0 = atomicAdd(&wc[d0], (uint32_t)__popc(p0));
+                    if (!any.value) wm[d0] = 0u;
+                }
+                o0 = __shfl_sync(0xffffffffu, o0, l0);
+                rk[i / 2] |= (o0 + __popc(p0 & lt)) << (16 * (i & 1));
                 __syncwarp();
             }
-            const int l0 = 31 - __clz(p0);
-            uint32_t o0 = 0;
-            if (lane == l0) {
-                o0 = atomicAdd(&wc[d0], (uint32_t)__popc(p0));
-                if (RANK == 3) wm[d0] = 0u;
-            }
-            o0 = __shfl_sync(0xffffffffu, o0, l0);
-            rk[i / 2] |= (o0 + __popc(p0 & lt)) << (16 * (i & 1));
-            __syncwarp();
-        }
+        };
+        if (match_any)
+            rank_columns(std::true_type{});
+        else
+            rank_columns(std::false_type{});
         __syncthreads();   // B1: every warp's digit counts are final
 
         if (tid < bins) {
@@ -317,7 +329,7 @@ __global__ void __launch_bounds__(BLOCK, (BLOCK >= 1024 ? 1 : 1024 / BLOCK))
 template <typename U, bool PAIRS, int BLOCK, int KPT, int D, int RANK>
 cudaError_t launch_reg_inst(size_t grid, int sms, cudaStream_t s, const RadixArgs& a, int pass) {
     auto kern = radix_onesweep_reg<U, PAIRS, BLOCK, KPT, D, RANK>;
-    const size_t smem = reg_smem_bytes(BLOCK, KPT, (int)sizeof(U), PAIRS, D, RANK);
+    const size_t smem = reg_smem_bytes(BLOCK, KPT, (int)sizeof(U), PAIRS, D, RANK == 1 ? 1 : 3);
     static int resident = 0;   // resident CTAs per SM
     if (resident == 0) {
         cudaError_t e = cudaSuccess;
@@ -333,17 +345,17 @@ cudaError_t launch_reg_inst(size_t grid, int sms, cudaStream_t s, const RadixArg
     size_t g = (size_t)sms * resident;
     if (g > grid) g = grid;
     if (g < 1) g = 1;
-    kern<<<(unsigned)g, BLOCK, smem, s>>>(a, pass);
-    return cudaGetLastError();
+    return launch_chain(kern, (unsigned)g, BLOCK, smem, s, a, pass);
 }
 
-// Rank modes of the register tile: 1 (match.any) and 3 (match masks); rank
-// mode 4 launches both per pass, as for the staged tile.
+// Rank modes of the register tile: 1 (match.any), 3 (match masks) and 4 (the
+// one the pass descriptor names).
 template <typename U, bool PAIRS, int B, int K>
 cudaError_t launch_reg_rank(int rank, size_t grid, int sms, cudaStream_t s, const RadixArgs& a, int pass) {
     if (a.d != 8) return cudaErrorInvalidConfiguration;
     if (rank == 1) return launch_reg_inst<U, PAIRS, B, K, 8, 1>(grid, sms, s, a, pass);
     if (rank == 3) return launch_reg_inst<U, PAIRS, B, K, 8, 3>(grid, sms, s, a, pass);
+    if (rank == 4) return launch_reg_inst<U, PAIRS, B, K, 8, 4>(grid, sms, s, a, pass);
     return cudaErrorInvalidConfiguration;
 }
 

@@ -149,6 +149,7 @@ __device__ __forceinline__ void hist_add_run(uint32_t* h, int cols, uint32_t dig
 
 template <typename U>
 __global__ void __launch_bounds__(kHistThreads) radix_histogram(RadixArgs a) {
+    chain_wait();
     extern __shared__ uint32_t s_h[];
     const int bins = 1 << a.d;
     const int cols = hist_cols(a.npass, a.d);
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(kHistThreads) radix_histogram(RadixArgs a) {
 // CTA publishes the bias), which K2 then uses in place of the raw counts.
 template <typename U, bool REBASE>
 __global__ void __launch_bounds__(kHistThreads) radix_histogram8(RadixArgs a) {
+    chain_wait();
     extern __shared__ uint32_t s_h[];
     constexpr int NP = (int)sizeof(U);
     constexpr int BINS = 256;
@@ -418,6 +420,7 @@ __global__ void __launch_bounds__(kHistThreads) radix_histogram8(RadixArgs a) {
 // keys (default 1/4, a.conc_first).  Both thresholds are tunable.
 
 static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int inplace) {
+    chain_wait();
     __shared__ unsigned long long s_scr[33];
     __shared__ int s_trivial[64];
     __shared__ int s_conc[64];
@@ -617,6 +620,7 @@ constexpr int onesweep_min_blocks(int block, int kpt) {
 
 template <typename U, bool PAIRS, int BLOCK, int KPT, int D, int RANK>
 __global__ void __launch_bounds__(BLOCK, onesweep_min_blocks(BLOCK, KPT)) radix_onesweep(RadixArgs a, int pass) {
+    chain_wait();
     constexpr int WARPS = BLOCK / 32;
     constexpr int TILE = BLOCK * KPT;
     constexpr int PER_MAX = ((1 << D) + BLOCK - 1) / BLOCK;
@@ -1046,6 +1050,7 @@ __device__ __forceinline__ void copy_reversed(const T* s, T* o, size_t n, size_t
 
 template <typename U>
 __global__ void __launch_bounds__(256) radix_fixup(RadixArgs a) {
+    chain_wait();
     const int fix = a.desc[a.npass].fixup;
     if (fix == FIX_NONE) return;
     U* o = (U*)a.out;

@@ -42,24 +42,24 @@ cudaError_t launch_radix_aux(int w, int which, size_t grid, size_t smem, cudaStr
         if (which == 3) {
             if (a.d != 8) return cudaErrorInvalidValue;
             if (w == 4)
-                radix_histogram8<uint32_t, true><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+                return launch_chain(radix_histogram8<uint32_t, true>, (unsigned)grid, kHistThreads, hs, s, a);
             else
-                radix_histogram8<uint64_t, true><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+                return launch_chain(radix_histogram8<uint64_t, true>, (unsigned)grid, kHistThreads, hs, s, a);
         } else if (a.d == 8 && w == 4)
-            radix_histogram8<uint32_t, false><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+            return launch_chain(radix_histogram8<uint32_t, false>, (unsigned)grid, kHistThreads, hs, s, a);
         else if (a.d == 8)
-            radix_histogram8<uint64_t, false><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+            return launch_chain(radix_histogram8<uint64_t, false>, (unsigned)grid, kHistThreads, hs, s, a);
         else if (w == 4)
-            radix_histogram<uint32_t><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+            return launch_chain(radix_histogram<uint32_t>, (unsigned)grid, kHistThreads, hs, s, a);
         else
-            radix_histogram<uint64_t><<<(unsigned)grid, kHistThreads, hs, s>>>(a);
+            return launch_chain(radix_histogram<uint64_t>, (unsigned)grid, kHistThreads, hs, s, a);
     } else if (which == 1) {
-        radix_scan_plan<<<1, 1024, 0, s>>>(a, inplace);
+        return launch_chain(radix_scan_plan, 1u, 1024u, (size_t)0, s, a, inplace);
     } else {
         if (w == 4)
-            radix_fixup<uint32_t><<<(unsigned)grid, 256, 0, s>>>(a);
+            return launch_chain(radix_fixup<uint32_t>, (unsigned)grid, 256u, (size_t)0, s, a);
         else
-            radix_fixup<uint64_t><<<(unsigned)grid, 256, 0, s>>>(a);
+            return launch_chain(radix_fixup<uint64_t>, (unsigned)grid, 256u, (size_t)0, s, a);
     }
     return cudaGetLastError();
 }

@@ -36,8 +36,7 @@ cudaError_t launch_onesweep_inst(size_t grid, int sms, cudaStream_t s, const Rad
     size_t g = (size_t)sms * resident;
     if (g > grid) g = grid;
     if (g < 1) g = 1;
-    kern<<<(unsigned)g, BLOCK, smem, s>>>(a, pass);
-    return cudaGetLastError();
+    return launch_chain(kern, (unsigned)g, BLOCK, smem, s, a, pass);
 }
 
 // Digit widths 4..11 with per-bit ballot ranking; shared match-mask ranking
