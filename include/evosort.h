@@ -471,7 +471,9 @@ typedef enum {
     EVOSORT_K_SMALL = 8,             /* one-CTA shared-memory sort of a small array */
     EVOSORT_K_DICT = 9,              /* few distinct keys: count (pass 0) and fill (pass 1) */
     EVOSORT_K_ORDERED = 10,          /* input in order: checked copy (pass 0), check (1), reversed copy (2) */
-    EVOSORT_K_RADIX_COUNT = 11       /* narrow key range: value count and fill (both launches in one record) */
+    EVOSORT_K_RADIX_COUNT = 11,      /* narrow key range: value count and fill (both launches in one record) */
+    EVOSORT_K_HYBRID = 12            /* partition sort of a large array: sample (pass 0), count, plan, step A (3),
+                                        count, scan, step B (6), groups, local sorts (8), clean-up */
 } evosort_kernel_kind;
 
 typedef struct {

@@ -186,6 +186,7 @@ static RadixLayout radix_layout(size_t n, int w, bool pairs, const Plan& pl) {
     L.off_counts = off;
     off = align_up(off + L.npass * bins * sizeof(unsigned long long), 256);
     L.off_range = off;   // RNG_WORDS range words (smallest / largest key, bias, flags)
+    static_assert(RNG_WORDS * sizeof(unsigned long long) + HYB_WORDS * 4 <= 256, "partition sort's control words");
     off = align_up(off + RNG_WORDS * sizeof(unsigned long long), 256);
     L.off_counts2 = off;   // digit counts of the rebased keys (8-bit digits only)
     off = align_up(off + (pl.digit_bits == 8 ? L.npass * bins * sizeof(unsigned long long) : 0), 256);
@@ -248,10 +249,37 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     a.range = (unsigned long long*)(base + L.off_range);
     a.counts2 = (unsigned long long*)(base + L.off_counts2);
     a.status = status;
+    a.hyb = nullptr;
     const int inplace = (in == out) ? 1 : 0;
 
-    cudaError_t e = cudaMemsetAsync(base, 0, L.zero_end, s);
+    // Partition sort first, where the plan asks for it: its tables lie in the
+    // look-back slots, which it leaves zeroed unless it sorted the array
+    const size_t hyb_bytes = hybrid_scratch_bytes(w, n);
+    const bool hybrid = pl.hybrid != HYBRID_OFF && !pairs && pl.digit_bits == 8 && n < (1ull << 31) &&
+                        hyb_bytes <= L.zero_end - L.off_lookback;
+    const bool ask = hybrid && pl.hybrid == HYBRID_SYNC;
+    cudaError_t e = cudaMemsetAsync(base, 0, ask ? L.off_lookback + hyb_bytes : L.zero_end, s);
     const int call = prof_call_begin(a.desc, L.npass + 1, s);
+    if (hybrid) {
+        uint32_t* ctl = (uint32_t*)(a.range + RNG_WORDS);   // fills up the range words' 256 bytes
+        if (e == cudaSuccess) e = launch_hybrid_sort(w, in, out, a.tmp, n, a.map, ctl, base + L.off_lookback,
+                                                     a.desc + L.npass, call, s);
+        if (!ask) {
+            a.hyb = ctl;
+        } else {
+            uint32_t said[HYB_WORDS] = {};
+            if (e == cudaSuccess) e = cudaMemcpyAsync(said, ctl, sizeof(said), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            const bool done = e == cudaSuccess && said[HYB_ON] != 0u && said[HYB_FAIL] == 0u;
+            if (done || e != cudaSuccess) {
+                prof_call_end(call, s, a.desc);
+                if (done) return EVOSORT_OK;
+                *err = std::string("partition sort: ") + cudaGetErrorString(e);
+                return EVOSORT_ERR_CUDA;
+            }
+            e = cudaMemsetAsync(base, 0, L.zero_end, s);
+        }
+    }
     const int sms = sm_count();
     const size_t hist_smem = (size_t)L.npass * ((size_t)1 << pl.digit_bits) * sizeof(uint32_t);
     size_t hist_grid = (n + 1024 * 16 - 1) / (1024 * 16);
@@ -592,6 +620,11 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
     }
     // dispatcher: tuned parameters for this input when the caller leaves the choice open
     evosort_params planned;
+    int hybrid = HYBRID_OFF;
+    if ((!p || (p->algo == EVOSORT_ALGO_AUTO && !p->digit_bits && !p->keys_per_thread && !p->block_size &&
+                !p->rank_mode && !p->pass_kernel && !p->adapt_later && !p->adapt_first)) &&
+        n >= kHybridMinAsync)
+        hybrid = HYBRID_ASYNC;
     if ((!p || p->algo == EVOSORT_ALGO_AUTO) && table_nonempty()) {
         void* st = p ? p->stream : nullptr;
         const bool desc = p && p->descending;
@@ -615,6 +648,9 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
             if (rco) return finish(rco, err);
             if (done) return EVOSORT_OK;
         }
+        // spread keys: the partition sort (an array of few values or in order
+        // has been sorted above, or proved to be neither)
+        hybrid = n >= kHybridMinSync && info.order == 0 && info.spread ? HYBRID_SYNC : HYBRID_OFF;
         if (p) {
             planned.stream = p->stream;
             planned.workspace = p->workspace;
@@ -651,6 +687,7 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
         return finish(EVOSORT_ERR_INVALID, "radix tile does not fit in shared memory (block_size x "
                                            "keys_per_thread too large for this key width and digit width)");
     cudaStream_t s = p ? (cudaStream_t)p->stream : nullptr;
+    pl.hybrid = hybrid;
 
     size_t need = 0;
     if (pl.algo == EVOSORT_ALGO_MERGE) {
@@ -896,6 +933,8 @@ size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
             }
             if (r.kind == EVOSORT_K_RADIX_FIXUP && r.pass >= 0 && r.pass < c.ndesc)
                 active = c.host_desc[r.pass].fixup != FIX_NONE;
+            if (r.kind == EVOSORT_K_HYBRID) active = c.host_desc[c.ndesc - 1].hybrid;
+            if (r.kind == EVOSORT_K_RADIX_HISTOGRAM && c.host_desc[c.ndesc - 1].hybrid) active = 0;
         }
         if (out && k < cap) {
             out[k].kind = r.kind;

@@ -28,7 +28,14 @@ struct Plan {
     int seg_warp_cap;         // segmented sort: warp tier below this length
     int small_cap;            // single-CTA path for lone arrays up to this size (1 = off)
     long long seg_giant;      // segmented sort: device-wide path above this length (-1 = off)
+    int hybrid = 0;           // partition sort (hybrid.cu) before the radix passes: a HYB_* mode
 };
+// The partition sort is tried only when the call leaves the choice to the
+// library.  HYBRID_ASYNC enqueues it and the radix kernels after it, which
+// return at once when it sorted the array; HYBRID_SYNC (the dispatcher's
+// calls, which have read a sample back already) reads its verdict back and
+// enqueues the radix kernels only when they are needed.
+enum : int { HYBRID_OFF = 0, HYBRID_ASYNC = 1, HYBRID_SYNC = 2 };
 
 // Single-CTA path for lone small arrays (Algorithm 5's small-array branch):
 // default and largest cut-over, in keys.
@@ -51,10 +58,14 @@ constexpr int kDictMax = 64;
 constexpr size_t kDictMinKeys = (size_t)1 << 16;
 // What a sample shows beyond its class: its distinct keys in the key map's
 // order (ascending) when there are at most kDictMax, and whether every
-// neighbour pair is non-decreasing (order 1), non-increasing (-1) or neither.
+// neighbour pair is non-decreasing (order 1), non-increasing (-1) or neither;
+// and whether the keys are spread as the partition sort (hybrid.cu) wants them:
+// no value holds a quarter of them, and either they span more than 24 bits
+// and no value repeats often, or most are of values that do.
 struct SampleInfo {
     std::vector<uint64_t> dict;
     int order = 0;
+    bool spread = false;   // worth trying the partition sort on
 };
 int classify_sample(const unsigned char* buf, size_t m, int dt, bool descending = false,
                     SampleInfo* info = nullptr);
@@ -104,6 +115,10 @@ class ProfScope {
 // Smallest sort that uses adaptive ranking (rank mode 4); smaller ones rank
 // with match masks only.
 constexpr size_t kAdaptMinKeys = (size_t)1 << 21;
+// Smallest sorts the partition sort is tried on: where the call waits for its
+// verdict, and where the radix kernels are enqueued after it in any case.
+constexpr size_t kHybridMinSync = (size_t)1 << 21;
+constexpr size_t kHybridMinAsync = (size_t)1 << 23;
 size_t radix_workspace_bytes(size_t n, int w, bool pairs, const Plan& pl);
 int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n, int dt,
                const Plan& pl, void* ws, size_t ws_bytes, cudaStream_t s, std::string* err);

@@ -71,11 +71,28 @@ int classify_sample(const unsigned char* buf, size_t m, int dt, bool descending,
     for (size_t i = 0; i < m; ++i) vary |= raw[i] ^ raw[0];
     std::vector<uint64_t> sorted(raw);
     std::sort(sorted.begin(), sorted.end());
-    const size_t distinct = std::unique(sorted.begin(), sorted.end()) - sorted.begin();
+    // runs of equal keys: their number (the first kDictMax + 1 values are kept
+    // at the front), the longest, and the keys in runs of four or more
+    const uint64_t least = sorted.front(), most = sorted.back();
+    size_t distinct = 0, longest = 0, often = 0;
+    for (size_t i = 0; i < m;) {
+        const uint64_t v = sorted[i];
+        size_t j = i + 1;
+        while (j < m && sorted[j] == v) ++j;
+        if (distinct <= (size_t)kDictMax) sorted[distinct] = v;   // distinct <= i
+        ++distinct;
+        longest = std::max(longest, j - i);
+        if (j - i >= 4) often += j - i;
+        i = j;
+    }
     if (info) {
         info->dict.clear();
         if (distinct <= (size_t)kDictMax) info->dict.assign(sorted.begin(), sorted.begin() + distinct);
         info->order = down == 0 ? 1 : (up == 0 ? -1 : 0);
+        // (the path's own sample decides in the end; this one only spares the
+        // launches and the wait where it is sure to say no)
+        const bool wide = ((most - least) >> 24) != 0;
+        info->spread = longest * 4 <= m && (wide ? longest * 128 <= m : often * 4 >= m);
     }
     // top-byte concentration: share of the sample in the most common top byte
     size_t top[256] = {0};

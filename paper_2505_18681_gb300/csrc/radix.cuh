@@ -21,6 +21,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "hybrid.cuh"
 
 namespace evosort {
 
@@ -45,7 +46,7 @@ struct PassDesc {
     int xout;     // apply from_ordered on store (last active pass)
     int fixup;    // used in the entry after the last pass
     int rank;     // adaptive ranking: the rank mode this pass runs with
-    int pad1;
+    int hybrid;   // used in the entry after the last pass: the partition sort sorted the array
 };
 
 struct RadixArgs {
@@ -73,6 +74,7 @@ struct RadixArgs {
     unsigned long long* range;  // RNG_WORDS words (RNG_*), zeroed with the counters
     unsigned long long* counts2;   // npass << d digit counts of the rebased keys
     uint32_t* status;
+    const uint32_t* hyb;    // control words of a partition sort launched before (hybrid.cuh), or null
 };
 
 // Range reduction ("rebase"): when the mapped keys span fewer 8-bit digits
@@ -271,6 +273,7 @@ template <typename U, bool REBASE>
 __global__ void __launch_bounds__(kHistThreads) radix_histogram8(RadixArgs a) {
     chain_wait();
     extern __shared__ uint32_t s_h[];
+    if (!REBASE && hybrid_done(a.hyb)) return;   // (K1b returns: K1 recorded nothing)
     constexpr int NP = (int)sizeof(U);
     constexpr int BINS = 256;
     constexpr int COLS = hist_cols(NP, 8);
@@ -425,6 +428,7 @@ static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int 
     __shared__ int s_trivial[64];
     __shared__ int s_conc[64];
     __shared__ double s_sq[32];
+    if (hybrid_done(a.hyb)) return;   // the descriptors stay zero: no pass and no fixup runs
     const int bins = 1 << a.d;
     const int per = (bins + 1023) / 1024;   // consecutive bins per thread (<= 2)
     // a rebased sort (K1b ran) plans from the digit counts of key - min
