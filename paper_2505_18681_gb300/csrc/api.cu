@@ -11,6 +11,7 @@
 #include "evosort.h"
 #include "api_internal.h"
 #include "closed_form.h"
+#include "fused.cuh"
 #include "radix_launch.cuh"
 
 namespace evosort {
@@ -153,6 +154,14 @@ ProfScope::ProfScope(int call, int kind, int pass, double bytes, uint64_t items,
     if (other) g_prof.push_back(ProfRecord{kind, pass, call, other, true, bytes, items, nullptr, nullptr});
 }
 
+// A step inside the launch whose scope was opened last: a record without a
+// time of its own, active or not as the pass descriptors say.
+void prof_inside(int call, int kind, int pass, double bytes, uint64_t items) {
+    if (!g_prof_on || call < 0) return;
+    std::lock_guard<std::mutex> lk(g_prof_mu);
+    g_prof.push_back(ProfRecord{kind, pass, call, 0, true, bytes, items, nullptr, nullptr});
+}
+
 ProfScope::~ProfScope() {
     if (idx_ < 0) return;
     std::lock_guard<std::mutex> lk(g_prof_mu);
@@ -252,6 +261,31 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
     a.hyb = nullptr;
     const int inplace = (in == out) ? 1 : 0;
 
+    // Mid-sized arrays: all passes in one launch (the partition sort, where it
+    // is asked for, comes first)
+    if (pl.fused && pl.hybrid == HYBRID_OFF && pl.digit_bits == 8 && n > kFusedMin && n <= fused_max_keys(w, pairs)) {
+        static_assert(8 * sizeof(unsigned long long) <= 256, "control words in the tile counters' room");
+        cudaError_t ef = cudaMemsetAsync(base, 0, L.off_counts, s);
+        const int fcall = prof_call_begin(a.desc, L.npass + 1, s);
+        const double bytes = 2.0 * (double)n * (w + (pairs ? 4 : 0));
+        if (ef == cudaSuccess) {
+            ProfScope ps(fcall, EVOSORT_K_RADIX_FUSED, -1, bytes, n, s);
+            for (int p = 0; p < L.npass; ++p) prof_inside(fcall, EVOSORT_K_RADIX_ONESWEEP, p, bytes, n);
+            prof_inside(fcall, EVOSORT_K_RADIX_FIXUP, L.npass, bytes, n);
+            ef = launch_radix_fused(w, in, out, vin, vout, n, a.map, (unsigned long long*)(base + L.off_tiles),
+                                    base + L.off_tmp, base + L.off_cbins, a.desc, status, s);
+        }
+        prof_call_end(fcall, s, a.desc);
+        if (ef == cudaSuccess) {
+            count_launches(1);
+            return EVOSORT_OK;
+        }
+        if (ef != cudaErrorCooperativeLaunchTooLarge && ef != cudaErrorNotSupported) {
+            *err = std::string("radix launch: ") + cudaGetErrorString(ef);
+            return EVOSORT_ERR_CUDA;
+        }
+        cudaGetLastError();   // the CTAs cannot all be resident: the chain of launches instead
+    }
     // Partition sort first, where the plan asks for it: its tables lie in the
     // look-back slots, which it leaves zeroed unless it sorted the array
     const size_t hyb_bytes = hybrid_scratch_bytes(w, n);
@@ -621,11 +655,22 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
     // dispatcher: tuned parameters for this input when the caller leaves the choice open
     evosort_params planned;
     int hybrid = HYBRID_OFF;
-    if ((!p || (p->algo == EVOSORT_ALGO_AUTO && !p->digit_bits && !p->keys_per_thread && !p->block_size &&
-                !p->rank_mode && !p->pass_kernel && !p->adapt_later && !p->adapt_first)) &&
-        n >= kHybridMinAsync)
-        hybrid = HYBRID_ASYNC;
-    if ((!p || p->algo == EVOSORT_ALGO_AUTO) && table_nonempty()) {
+    const bool automatic = !p || p->algo == EVOSORT_ALGO_AUTO;
+    const bool own_genes = p && (p->keys_per_thread || p->block_size || p->rank_mode || p->pass_kernel ||
+                                 p->adapt_later || p->adapt_first);   // the pass kernels are the caller's choice
+    if (automatic && !own_genes && !(p && p->digit_bits) && n >= kHybridMinAsync) hybrid = HYBRID_ASYNC;
+    bool fused = !own_genes;
+    // below kDictMinKeys the class only picks a tile, which the one-launch sort
+    // does not use (unless the table may pick the mergesort): no sample then.
+    // (While a stream is captured the sample stays, and refuses the call.)
+    auto needs_no_sample = [&]() {
+        if (!fused || n >= kDictMinKeys || n > fused_max_keys(w, pairs) || n <= kFusedMin) return false;
+        if (table_has_algo(dt, EVOSORT_ALGO_MERGE)) return false;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        return cudaStreamIsCapturing(p ? (cudaStream_t)p->stream : nullptr, &cap) == cudaSuccess &&
+               cap == cudaStreamCaptureStatusNone;
+    };
+    if (automatic && table_nonempty() && !needs_no_sample()) {
         void* st = p ? p->stream : nullptr;
         const bool desc = p && p->descending;
         int cls = EVOSORT_CLASS_RANDOM;
@@ -650,6 +695,7 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
         }
         // spread keys: the partition sort (an array of few values or in order
         // has been sorted above, or proved to be neither)
+        fused = true;   // (the table's tile is for the chain of launches)
         hybrid = n >= kHybridMinSync && info.order == 0 && info.spread ? HYBRID_SYNC : HYBRID_OFF;
         if (p) {
             planned.stream = p->stream;
@@ -688,6 +734,7 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
                                            "keys_per_thread too large for this key width and digit width)");
     cudaStream_t s = p ? (cudaStream_t)p->stream : nullptr;
     pl.hybrid = hybrid;
+    pl.fused = fused;
 
     size_t need = 0;
     if (pl.algo == EVOSORT_ALGO_MERGE) {
@@ -919,7 +966,7 @@ size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
             launch_ms = 0.f;
             cudaEventElapsedTime(&launch_ms, r.e0, r.e1);
         }
-        float ms = launch_ms;
+        float ms = r.same && r.rank == 0 ? 0.f : launch_ms;   // (a step inside a launch has no time of its own)
         int active = 1;
         const ProfCall& c = g_prof_calls[r.call];
         if (c.copied) cudaEventSynchronize(c.copied);
@@ -928,7 +975,7 @@ size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
                 active = c.host_desc[r.pass].active && (r.rank == 0 || c.host_desc[r.pass].rank == r.rank);
                 // one launch for both variants: its time goes to the one that
                 // ran (to the first if the pass was skipped)
-                const bool both = r.same || (i + 1 < g_prof.size() && g_prof[i + 1].same);
+                const bool both = r.rank != 0 && (r.same || (i + 1 < g_prof.size() && g_prof[i + 1].same));
                 if (both && !active && (r.same || c.host_desc[r.pass].active)) ms = 0.f;
             }
             if (r.kind == EVOSORT_K_RADIX_FIXUP && r.pass >= 0 && r.pass < c.ndesc)

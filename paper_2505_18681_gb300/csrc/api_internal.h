@@ -28,7 +28,8 @@ struct Plan {
     int seg_warp_cap;         // segmented sort: warp tier below this length
     int small_cap;            // single-CTA path for lone arrays up to this size (1 = off)
     long long seg_giant;      // segmented sort: device-wide path above this length (-1 = off)
-    int hybrid = 0;           // partition sort (hybrid.cu) before the radix passes: a HYB_* mode
+    int hybrid = 0;           // partition sort (hybrid.cu) before the radix passes: a HYBRID_* mode
+    bool fused = false;       // mid-sized radix sorts in one launch (fused.cu) where they fit
 };
 // The partition sort is tried only when the call leaves the choice to the
 // library.  HYBRID_ASYNC enqueues it and the radix kernels after it, which
@@ -51,6 +52,7 @@ uint32_t wait_limit();
 void set_error(const std::string& msg);
 void default_radix_plan(int dt, Plan* pl, size_t n = 0);
 bool table_nonempty();
+bool table_has_algo(int dt, int algo);   // some entry of the key type names this algorithm
 // Largest distinct-value count of the dictionary path, and the smallest
 // array it and the ordered path are tried on (below that the radix sort's
 // fixed cost is small).
@@ -99,6 +101,7 @@ uint32_t* status_word(std::string* err);
 
 struct PassDesc;
 bool prof_enabled();
+void prof_inside(int call, int kind, int pass, double bytes, uint64_t items);
 int prof_call_begin(const PassDesc* dev_desc, int ndesc, cudaStream_t s);
 void prof_call_end(int call, cudaStream_t s, const PassDesc* dev_desc);
 // Records a CUDA event pair around one launch while instrumentation is on.
@@ -115,6 +118,9 @@ class ProfScope {
 // Smallest sort that uses adaptive ranking (rank mode 4); smaller ones rank
 // with match masks only.
 constexpr size_t kAdaptMinKeys = (size_t)1 << 21;
+// Smallest radix sort that goes into one launch (up to fused_max_keys); below
+// it a chain of launches has hardly anything to move either.
+constexpr size_t kFusedMin = 2048;
 // Smallest sorts the partition sort is tried on: where the call waits for its
 // verdict, and where the radix kernels are enqueued after it in any case.
 constexpr size_t kHybridMinSync = (size_t)1 << 21;

@@ -149,6 +149,13 @@ bool table_nonempty() {
     return !g_tab.empty();
 }
 
+bool table_has_algo(int dt, int algo) {
+    std::lock_guard<std::mutex> lk(g_tab_mu);
+    for (const auto& x : g_tab)
+        if (x.dt == dt && x.p.algo == algo) return true;
+    return false;
+}
+
 // Class of keys[0..n) (a device array) from a strided sample, read in the
 // order of the sort's direction (synchronises the stream).
 evosort_status classify_device(const void* keys, size_t n, int dt, void* stream, bool descending,
