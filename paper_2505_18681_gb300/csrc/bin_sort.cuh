@@ -31,7 +31,6 @@ namespace evosort {
 
 constexpr int kBinMax = 1 << 15;     // most bins
 constexpr int kBinThreadKeys = 31;   // longest bin one thread sorts (2^k - 1)
-constexpr int kBinWide = 12;         // bins per thread of block_bin_sort_wide
 constexpr int kBinWarpKeys = 16;     // keys per lane of the warp sort
 
 // Bytes of the second buffer of n keys: the words of the bins, or the merge
@@ -94,6 +93,15 @@ __device__ __forceinline__ void cut_range_near(unsigned long long width, uint32_
 __device__ __forceinline__ uint32_t part_start(uint32_t j, uint32_t mult) {
     return (uint32_t)((((unsigned long long)j << 32) + mult - 1ull) / mult);
 }
+
+// Position of a key in [lo, lo + width].
+template <typename U>
+struct KeyPosition {
+    static constexpr bool linear = true;   // few enough values: one per bin
+    U lo;
+    int lz;
+    __device__ __forceinline__ uint32_t operator()(U k) const { return norm32((U)(k - lo), lz); }
+};
 
 template <typename U, int NT>
 struct BinShared {
@@ -160,6 +168,29 @@ __device__ __forceinline__ void bin_insertion(U* k, int c) {
     }
 }
 
+// The same for keys with their input positions (x), in the order (key,
+// position): equal keys keep their input order.
+template <typename U>
+__device__ __forceinline__ void bin_insertion_indexed(U* k, uint16_t* x, int c) {
+    for (int i = 1; i < c; ++i) {
+        const U a = k[i];
+        const uint16_t xa = x[i];
+        int j = i;
+        while (j > 0) {
+            const U y = k[j - 1];
+            const uint16_t xy = x[j - 1];
+            if (!(y > a || (y == a && xy > xa))) break;
+            k[j] = y;
+            x[j] = xy;
+            --j;
+        }
+        if (j < i) {
+            k[j] = a;
+            x[j] = xa;
+        }
+    }
+}
+
 // Sort of k[0..c), c <= 32 * kBinWarpKeys, by one warp.
 template <typename U>
 __device__ __noinline__ void bin_warp_sort(U* k, int c) {
@@ -220,7 +251,8 @@ __device__ __forceinline__ void bin_zero(U* k1) {
 }
 
 // The same sort with 32-bit counters and any distribution of the keys, which
-// lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per thread.
+// lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per
+// thread: the words of block_bin_sort, so that k1 is as large as there.
 template <typename U, int NT, int KPT, int BPT>
 __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, U* k0, U* k1,
                                                      BinShared<U, NT>& sh) {
@@ -301,15 +333,19 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
 // Sorts the n keys that the CTA's NT threads hold in registers (key i of a
 // thread is element i * NT + thread; elements from n on are ignored), all in
 // [lo, lo + width].  The words in k1 are zero (bin_zero) and every thread
-// knows it.  WPT words of four bins per thread; (lz, mult) from
-// cut_range(width, 4 * WPT * NT).  k0 holds n keys, k1 bin_scratch_bytes(n, w,
+// knows it.  WPT words of four bins per thread: bin = umulhi(position(key),
+// mult), where position is a KeyPosition (mult and lz from cut_range(width, 4 *
+// WPT * NT)) or any other function that never falls as the keys rise.  k0 holds n keys, k1 bin_scratch_bytes(n, w,
 // WPT * NT) bytes, both 16-byte aligned; n < 2^14.  placed() runs once the
 // registers' keys are in shared memory (the caller may reload them, all of
 // them).  Returns the sorted array (k0 or k1), complete for every thread.
-template <typename U, int NT, int KPT, int WPT, typename F>
-__device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U lo, unsigned long long width, int lz,
-                                                   uint32_t mult, U* k0, U* k1, BinShared<U, NT>& sh,
-                                                   const F& placed) {
+// With IDX, x0 receives the input position of each sorted key, equal keys in
+// input order; where the stretches do not separate the keys it returns null
+// and has sorted nothing.
+template <typename U, int NT, int KPT, int WPT, bool IDX = false, typename P, typename F>
+__device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U lo, unsigned long long width,
+                                                   const P& position, uint32_t mult, U* k0, U* k1,
+                                                   BinShared<U, NT>& sh, const F& placed, uint16_t* x0 = nullptr) {
     static_assert(WPT % 8 == 4 && 4 * WPT * NT <= kBinMax && KPT * NT < (1 << 14), "words per thread");
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -327,7 +363,7 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
             for (int i = c; i < c + 4 && i < KPT; ++i) {
                 if (i * NT + tid < n) {
                     // (in range for every key of [lo, lo + width]; never out of the array for any other)
-                    const uint32_t b = min(__umulhi(norm32((U)(key[i] - lo), lz), mult), (uint32_t)(4 * WPT * NT - 1));
+                    const uint32_t b = min(__umulhi(position(key[i]), mult), (uint32_t)(4 * WPT * NT - 1));
                     const uint32_t old = atomicAdd(&words[b >> 2], __funnelshift_l(0u, 1u, 8u * b));   // by 8 (b mod 4)
                     br[i] = b << 8 | (__funnelshift_r(old, 0u, 8u * b) & 0xFFu);
                 }
@@ -366,13 +402,17 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
         const uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
         run += __reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);
         if (heavy || __reduce_add_sync(0xffffffffu, v) != (uint32_t)n) {   // the same for every thread
+            if constexpr (IDX) {
+                return nullptr;
+            } else {
 #pragma unroll
-            for (int i = 0; i < KPT; ++i)
-                if (i * NT + tid < n) k0[i * NT + tid] = key[i];
-            __syncthreads();
-            const U* r = block_bin_sort_wide<U, NT, KPT, kBinWide>(n, lo, width, k0, k1, sh);
-            placed();
-            return r;
+                for (int i = 0; i < KPT; ++i)
+                    if (i * NT + tid < n) k0[i * NT + tid] = key[i];
+                __syncthreads();
+                const U* r = block_bin_sort_wide<U, NT, KPT, WPT>(n, lo, width, k0, k1, sh);
+                placed();
+                return r;
+            }
         }
     }
 #pragma unroll
@@ -401,14 +441,16 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
                 if (i * NT + tid < n) {
                     const uint32_t b = br[i] >> 8, w = words[b >> 2];
                     const uint32_t before = ((w << 6) >> (6u * (b & 3u))) & 0x3Fu;   // keys of the word's earlier bins
-                    k0[(w >> 18) + before + (br[i] & 0xFFu)] = key[i];
+                    const uint32_t at = (w >> 18) + before + (br[i] & 0xFFu);
+                    k0[at] = key[i];
+                    if (IDX) x0[at] = (uint16_t)(i * NT + tid);
                 }
             }
         }
     }
     placed();
     __syncthreads();
-    if (width < (unsigned long long)(4 * WPT * NT)) return k0;   // a bin holds one value
+    if (!IDX && P::linear && width < (unsigned long long)(4 * WPT * NT)) return k0;   // a bin holds one value
 
     // ---- words with several keys in a bin: first the pairs, which are most of
     // them, so that a warp's lanes stay together; then the longer ones
@@ -420,7 +462,15 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
         const uint32_t at = own[q] >> 18, next = q + 1 < WPT ? own[q + 1] >> 18 : run;
         if (next - at == 2u) {
             const U a = k0[at], b = k0[at + 1];
-            if (b < a) {
+            if (IDX) {
+                const uint16_t xa = x0[at], xb = x0[at + 1];
+                if (b < a || (b == a && xb < xa)) {
+                    k0[at] = b;
+                    k0[at + 1] = a;
+                    x0[at] = xb;
+                    x0[at + 1] = xa;
+                }
+            } else if (b < a) {
                 k0[at] = b;
                 k0[at + 1] = a;
             }
@@ -432,7 +482,10 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
         const int q = __ffs((int)more) - 1;
         more &= more - 1u;
         const uint32_t at = own[q] >> 18, next = q + 1 < WPT ? own[q + 1] >> 18 : run;
-        bin_insertion(k0 + at, (int)(next - at));
+        if (IDX)
+            bin_insertion_indexed(k0 + at, x0 + at, (int)(next - at));
+        else
+            bin_insertion(k0 + at, (int)(next - at));
     }
     __syncthreads();
     return k0;

@@ -90,12 +90,14 @@ __device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int
         bin_zero<kCtaThreads, kCtaFewWords>(k1);
         __syncthreads();
         cut_range_near(width, (uint32_t)(4 * kCtaFewWords * kCtaThreads), &lz, &mult);
-        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaFewWords>(key, n, lo, width, lz, mult, k0, k1, sh.bin, []() {});
+        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaFewWords>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult,
+                                                                              k0, k1, sh.bin, []() {});
     } else {
         bin_zero<kCtaThreads, kCtaWords>(k1);
         __syncthreads();
         cut_range_near(width, (uint32_t)(4 * kCtaWords * kCtaThreads), &lz, &mult);
-        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaWords>(key, n, lo, width, lz, mult, k0, k1, sh.bin, []() {});
+        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaWords>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult,
+                                                                              k0, k1, sh.bin, []() {});
     }
     for (int i = threadIdx.x; i < n; i += kCtaThreads) store(i, r[i]);
     __syncthreads();

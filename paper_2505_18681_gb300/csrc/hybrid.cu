@@ -1056,7 +1056,7 @@ __global__ void __launch_bounds__(kHybThreads, 2) hybrid_local(HybArgs a) {
             load(s_q[cur ^ 1]);
         } else if (len > 0) {
             const U* r = block_bin_sort<U, kHybThreads, KPT, kHybLocalWords>(
-                key, (int)len, (U)q.lo, q.width, q.lz, q.mult, k0, k1, s_cta.bin, [&]() { load(s_q[cur ^ 1]); });
+                key, (int)len, (U)q.lo, q.width, KeyPosition<U>{(U)q.lo, q.lz}, q.mult, k0, k1, s_cta.bin, [&]() { load(s_q[cur ^ 1]); });
             U* const mine = out + q.start + tid;
             const U* const from = r + tid;
             if (plain) {
