@@ -106,7 +106,7 @@ struct KeyPosition {
 template <typename U, int NT>
 struct BinShared {
     U mn[NT / 32], mx[NT / 32];
-    uint32_t wsum[NT / 32];
+    uint32_t wsum[NT / 32 + 1];
     uint32_t nlist, big;
     uint32_t list[512];   // bins left to the warps: first position | length << 16
 };
@@ -340,9 +340,9 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
 // registers' keys are in shared memory (the caller may reload them, all of
 // them).  Returns the sorted array (k0 or k1), complete for every thread.
 // With IDX, x0 receives the input position of each sorted key, equal keys in
-// input order; where the stretches do not separate the keys it returns null
-// and has sorted nothing.
-template <typename U, int NT, int KPT, int WPT, bool IDX = false, typename P, typename F>
+// input order.  With OWN it returns null, and has sorted nothing, where the
+// stretches do not separate the keys: the caller has its own way then.
+template <typename U, int NT, int KPT, int WPT, bool IDX = false, bool OWN = IDX, typename P, typename F>
 __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U lo, unsigned long long width,
                                                    const P& position, uint32_t mult, U* k0, U* k1,
                                                    BinShared<U, NT>& sh, const F& placed, uint16_t* x0 = nullptr) {
@@ -396,13 +396,14 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
     }
     if (lane == 31) sh.wsum[warp] = inc;
     // a word's counts must stay below 64 in all: bins below 16
-    const bool heavy = __syncthreads_or((any & 0xF0F0F0F0u) != 0u);
+    // (of equal keys every one has to be put in order if there are positions)
+    const bool heavy = __syncthreads_or((any & (IDX ? 0xF8F8F8F8u : 0xF0F0F0F0u)) != 0u);
     uint32_t run = inc - sum;
     {
         const uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
         run += __reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);
         if (heavy || __reduce_add_sync(0xffffffffu, v) != (uint32_t)n) {   // the same for every thread
-            if constexpr (IDX) {
+            if constexpr (OWN) {
                 return nullptr;
             } else {
 #pragma unroll

@@ -8,8 +8,9 @@
 // (bin_sort.cuh), mapped back and stored.  Key/value sorts order the keys with
 // their input positions, so equal keys keep their input order and each value
 // is fetched once at the end (the stable argsort); where the range does not
-// separate the keys they take the merge sort of Algorithm 3 (insertion-sorted
-// base runs, then pairwise merges with merge-path splits).
+// separate the keys they take stable radix passes over the range in shared
+// memory, or the merge sort of Algorithm 3 (insertion-sorted base runs, then
+// pairwise merges with merge-path splits), whichever has fewer rounds.
 //
 // What bounds it is latency: some ten barriers and the accesses between them.
 // The merge sort had six to nine rounds, each a binary search and a serial
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
     uint32_t* v0 = (uint32_t*)((char*)k1 + small_up(bin_scratch_bytes(n, (int)sizeof(U), WPT * NT)));
     uint32_t* v1 = v0 + (PAIRS ? n : 0);
     uint16_t* x0 = (uint16_t*)v1;
+    uint16_t* counts = (uint16_t*)(v1 + (PAIRS ? n : 0));   // of the radix passes
     const int tid = threadIdx.x;
     U key[KPT];
 #pragma unroll
@@ -94,6 +96,13 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
     block_extent<U, NT, KPT>(key, n, sh, &lo, &hi);   // (its barrier also ends the clearing)
     const unsigned long long width = (unsigned long long)(U)(hi - lo);
     const U* ks;
+    if (width == 0) {   // equal keys: in order as they are
+        for (int i = tid; i < n; i += NT) {
+            out[i] = map_inv(lo, map);
+            if (PAIRS) vout[i] = v0[i];   // (written before block_extent's barrier)
+        }
+        return;
+    }
     if (FLT) {
         // smallest and largest finite value, then the same bins by value
         __shared__ float s_f[2][NT / 32];
@@ -127,24 +136,32 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
         const float range = 0.5f * b - 0.5f * a;   // negative or NaN if no value is finite: one bin
         const float scale = range > 0.f ? fminf(4294967040.f / range, FLT_MAX) : 0.f;
         const ValuePosition<U> pos{map, 0.5f * (desc ? b : a), scale, desc};
-        ks = block_bin_sort<U, NT, KPT, WPT, PAIRS>(key, n, lo, width, pos, (uint32_t)(4 * WPT * NT), k0, k1, sh,
-                                                    []() {}, x0);
+        ks = block_bin_sort<U, NT, KPT, WPT, PAIRS, true>(key, n, lo, width, pos, (uint32_t)(4 * WPT * NT), k0, k1, sh,
+                                                          []() {}, x0);
     } else {
         int lz;
         uint32_t mult;
         cut_range_near(width, (uint32_t)(4 * WPT * NT), &lz, &mult);
-        ks = block_bin_sort<U, NT, KPT, WPT, PAIRS>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult, k0, k1, sh,
-                                                    []() {}, x0);
+        ks = block_bin_sort<U, NT, KPT, WPT, PAIRS, true>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult, k0, k1,
+                                                          sh, []() {}, x0);
     }
     const uint32_t* vs = v0;
     bool by_position = true;
-    if (PAIRS && ks == nullptr) {
+    if (ks == nullptr) {
+        // frequent values, or keys crowded into a small part of their range:
+        // radix passes over the range, or the merge rounds where they are fewer
+        // (a pass takes about as long as a round: 1.2 us at 1,000 keys)
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < KPT; ++i)
             if (i * NT + tid < n) k0[i * NT + tid] = key[i];
         __syncthreads();
-        const int which = smem_merge_sort<U, PAIRS, kSmallRun>(k0, k1, v0, v1, n, tins);
+        const int passes = (64 - __clzll((long long)width) + 7) / 8;
+        int rounds = 1;
+        while ((kSmallRun << rounds) < n) ++rounds;
+        const int which = passes <= rounds
+                              ? smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, passes, counts, sh.wsum)
+                              : smem_merge_sort<U, PAIRS, kSmallRun>(k0, k1, v0, v1, n, tins);
         ks = which ? k1 : k0;
         vs = which ? v1 : v0;
         by_position = false;
@@ -165,7 +182,7 @@ cudaError_t launch_small_shape(const void* in, void* out, const uint32_t* vin, u
     auto kern = small_sort_kernel<U, PAIRS, FLT, KPT, WPT>;
     auto bytes = [](int m) {
         return small_up(m * sizeof(U)) + small_up(bin_scratch_bytes(m, (int)sizeof(U), WPT * kSmallThreads)) +
-               (PAIRS ? (size_t)m * 8 : 0);
+               (PAIRS ? (size_t)m * 8 : 0) + (size_t)kSmallThreads / 32 * 512;
     };
     static bool configured = false;
     if (!configured) {

@@ -159,6 +159,81 @@ __device__ int smem_merge_sort(U* k0, U* k1, uint32_t* v0, uint32_t* v1, int len
 }
 
 // ---------------------------------------------------------------------------
+// CTA radix sort (Algorithms 4a/4b in one CTA): stable LSD passes over 8-bit
+// digits of k - lo, from k0/v0 through k1/v1, for len <= 32 * COLS keys per
+// warp.  passes: digits of the keys' range.  counts: NT / 32 x 256 16-bit
+// counters.  Returns 0 if the result is in k0/v0, 1 if in k1/v1.  All threads
+// of the CTA must call it.
+// ---------------------------------------------------------------------------
+template <typename U, bool PAIRS, int NT, int COLS>
+__device__ __noinline__ int smem_radix_sort(U* k0, U* k1, uint32_t* v0, uint32_t* v1, int len, U lo, int passes,
+                                            uint16_t* counts, uint32_t* scratch) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cols = (len + NT - 1) / NT;   // columns of 32 keys per warp, consecutive in the array
+    const int wofs = warp * 32 * cols + lane;
+    const uint32_t lt = lanemask_lt();
+    uint16_t* const mine = counts + warp * 256;
+    for (int p = 0; p < passes; ++p) {
+        for (int i = lane; i < 128; i += 32) ((uint32_t*)mine)[i] = 0u;
+        __syncwarp();
+        U key[COLS];
+        uint32_t val[PAIRS ? COLS : 1];
+        uint32_t dr[COLS];   // digit | rank << 16
+#pragma unroll
+        for (int i = 0; i < COLS; ++i) {
+            if (i < cols) {
+                const int s = wofs + 32 * i;
+                const bool have = s < len;
+                key[i] = have ? k0[s] : (U)0;
+                if (PAIRS) val[PAIRS ? i : 0] = have ? v0[s] : 0u;
+                const uint32_t d = digit_of((U)(key[i] - lo), 8 * p, 0xFFu);
+                uint32_t peers = __ballot_sync(0xffffffffu, have);   // lanes with the same digit
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    const uint32_t m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                    peers &= (d >> b) & 1u ? m : ~m;
+                }
+                uint32_t before = 0;
+                const int leader = 31 - __clz((int)peers);
+                if (have && lane == leader) {
+                    before = mine[d];
+                    mine[d] = (uint16_t)(before + __popc(peers));
+                }
+                before = __shfl_sync(0xffffffffu, before, have ? leader : lane);
+                dr[i] = d | (before + (uint32_t)__popc(peers & lt)) << 16;
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        uint32_t sum = 0, tot;
+        if (tid < 256)
+            for (int w = 0; w < NW; ++w) sum += counts[w * 256 + tid];
+        uint32_t run = block_exclusive_scan<NT>(sum, scratch, &tot);
+        if (tid < 256) {
+            for (int w = 0; w < NW; ++w) {
+                const uint32_t c = counts[w * 256 + tid];
+                counts[w * 256 + tid] = (uint16_t)run;
+                run += c;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < COLS; ++i) {
+            if (i < cols && wofs + 32 * i < len) {
+                const uint32_t at = mine[dr[i] & 0xFFFFu] + (dr[i] >> 16);
+                k1[at] = key[i];
+                if (PAIRS) v1[at] = val[PAIRS ? i : 0];
+            }
+        }
+        __syncthreads();
+        U* t = k0; k0 = k1; k1 = t;
+        uint32_t* tv = v0; v0 = v1; v1 = tv;
+    }
+    return passes & 1;
+}
+
+// ---------------------------------------------------------------------------
 // Warp bitonic sort of 32*KW keys, ascending.  Lane L holds keys
 // [L*KW, (L+1)*KW) of the sequence in k[0..KW) (blocked layout); KW is a power
 // of two.  Not stable (used for keys-only sorts, where equal keys are
