@@ -24,6 +24,8 @@
 // still the merge sort of Algorithm 3, so any input is sorted in bounded time.
 #pragma once
 
+#include <cfloat>
+
 #include "common.cuh"
 #include "smem_sort.cuh"
 
@@ -102,6 +104,102 @@ struct KeyPosition {
     int lz;
     __device__ __forceinline__ uint32_t operator()(U k) const { return norm32((U)(k - lo), lz); }
 };
+
+// Key maps of a first load and a last store, as function objects: integers are
+// mapped by one xor (which is its own inverse), floats by the general map.
+template <typename U>
+struct XorMap {
+    static constexpr bool is_float = false;
+    U c;
+    __device__ __forceinline__ explicit XorMap(const KeyMap& m) : c((U)(m.s ^ m.x)) {}
+    __device__ __forceinline__ U operator()(U k) const { return k ^ c; }
+};
+template <typename U>
+struct FloatIn {
+    KeyMap m;
+    __device__ __forceinline__ explicit FloatIn(const KeyMap& k) : m(k) {}
+    __device__ __forceinline__ U operator()(U k) const { return map_fwd(k, m); }
+};
+template <typename U>
+struct GeneralOut {   // any key type
+    static constexpr bool is_float = false;
+    KeyMap m;
+    __device__ __forceinline__ explicit GeneralOut(const KeyMap& k) : m(k) {}
+    __device__ __forceinline__ U operator()(U k) const { return map_inv(k, m); }
+};
+template <typename U>
+struct FloatOut : GeneralOut<U> {
+    static constexpr bool is_float = true;
+    __device__ __forceinline__ explicit FloatOut(const KeyMap& k) : GeneralOut<U>(k) {}
+    __device__ __forceinline__ bool descending() const { return this->m.x != 0; }
+};
+
+// Position of a float key by its value: (value - smallest) * scale.  Floats of
+// an even spread crowd into the few bit patterns of the largest exponents, so
+// equal stretches of the mapped keys would leave most bins empty; equal
+// stretches of the values do not.  Rounding keeps the order: subtraction,
+// multiplication and the narrowing of doubles never turn two values around.
+// NaNs, which have no value, go to their end of the order, infinities and
+// values outside the range clamp.  (34.9e6 doubles in 3,000 segments: 2.41 ms
+// by equal stretches of the mapped keys, 0.79 ms by value.)
+__device__ __forceinline__ float float_of(uint32_t bits) { return __uint_as_float(bits); }
+__device__ __forceinline__ float float_of(uint64_t bits) {
+    return __double2float_rn(__longlong_as_double((long long)bits));
+}
+template <typename U, typename MO>
+struct ValuePosition {
+    static constexpr bool linear = false;
+    MO out;
+    float low, scale;   // of half the value, so that the widest range stays finite
+    bool descending;
+    // a, b: smallest and largest value of the range (a > b if there is none)
+    __device__ __forceinline__ ValuePosition(const MO& o, float a, float b, bool desc)
+        : out(o), low(0.5f * (desc ? b : a)), scale(0.f), descending(desc) {
+        const float range = 0.5f * b - 0.5f * a;
+        if (range > 0.f) scale = fminf(4294967040.f / range, FLT_MAX);
+    }
+    __device__ __forceinline__ uint32_t operator()(U k) const {
+        const float f = float_of(out(k));
+        if (f != f) return descending ? 0u : 0xFFFFFFFFu;
+        const float h = 0.5f * f;
+        const float x = (descending ? low - h : h - low) * scale;
+        return x <= 0.f ? 0u : (x >= 4294967040.f ? 0xFFFFFFFFu : (uint32_t)x);
+    }
+};
+// The position over the finite values of the CTA's keys (element i * NT +
+// thread < n, mapped; out maps back).
+template <typename U, int NT, int KPT, typename MO>
+__device__ __forceinline__ ValuePosition<U, MO> block_value_position(const U (&key)[KPT], int n, const MO& out, bool desc,
+                                                                     float (&s_f)[2][NT / 32]) {
+    const int tid = threadIdx.x;
+    float a = INFINITY, b = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        if (i * NT + tid < n) {
+            const float f = float_of(out(key[i]));
+            if (fabsf(f) < INFINITY) {
+                a = fminf(a, f);
+                b = fmaxf(b, f);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a = fminf(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if ((tid & 31) == 0) {
+        s_f[0][tid >> 5] = a;
+        s_f[1][tid >> 5] = b;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+        a = fminf(a, s_f[0][w]);
+        b = fmaxf(b, s_f[1][w]);
+    }
+    return ValuePosition<U, MO>(out, a, b, desc);
+}
 
 template <typename U, int NT>
 struct BinShared {

@@ -48,56 +48,48 @@ struct CtaShared {
     BinShared<U, kCtaThreads> bin;
     uint32_t scan[kCtaWarps + 1];
     uint32_t next, end, below, above, longest;
+    float value[2][kCtaWarps];
     int active[sizeof(U)];
 };
 
-// Key maps of the first load and the last store: integers are mapped by one
-// xor (which is its own inverse), floats by the general map.
-template <typename U>
-struct XorMap {
-    U c;
-    __device__ __forceinline__ explicit XorMap(const KeyMap& m) : c((U)(m.s ^ m.x)) {}
-    __device__ __forceinline__ U operator()(U k) const { return k ^ c; }
-};
-template <typename U>
-struct FloatIn {
-    KeyMap m;
-    __device__ __forceinline__ explicit FloatIn(const KeyMap& k) : m(k) {}
-    __device__ __forceinline__ U operator()(U k) const { return map_fwd(k, m); }
-};
-template <typename U>
-struct FloatOut {
-    KeyMap m;
-    __device__ __forceinline__ explicit FloatOut(const KeyMap& k) : m(k) {}
-    __device__ __forceinline__ U operator()(U k) const { return map_inv(k, m); }
-};
 struct AsIs {
     template <typename U>
     __device__ __forceinline__ U operator()(U k) const { return k; }
 };
 
-// Local sort of n <= cta_cap() keys held in registers (mapped), in [lo, lo +
-// width]; store(position, key) receives the sorted keys.
-template <typename U, typename S>
-__device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int n, U lo, unsigned long long width,
-                                               unsigned char* smem, CtaShared<U>& sh, const S& store) {
+// Local sort of n <= cta_cap() keys held in registers (mapped); out maps back,
+// store(position, key) receives the sorted keys, still mapped.  Bins by the
+// keys' range, or by their values' for floats.
+template <typename U, typename MO, typename S>
+__device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int n, const MO& out, unsigned char* smem,
+                                               CtaShared<U>& sh, const S& store) {
+    constexpr int KPT = cta_kpt<U>();
     U* k0 = (U*)smem;
     U* k1 = k0 + cta_cap<U>();
-    int lz;
-    uint32_t mult;
-    const U* r;
-    if (n <= kCtaFewKeys) {
+    if (n <= kCtaFewKeys)
         bin_zero<kCtaThreads, kCtaFewWords>(k1);
-        __syncthreads();
-        cut_range_near(width, (uint32_t)(4 * kCtaFewWords * kCtaThreads), &lz, &mult);
-        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaFewWords>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult,
-                                                                              k0, k1, sh.bin, []() {});
-    } else {
+    else
         bin_zero<kCtaThreads, kCtaWords>(k1);
-        __syncthreads();
-        cut_range_near(width, (uint32_t)(4 * kCtaWords * kCtaThreads), &lz, &mult);
-        r = block_bin_sort<U, kCtaThreads, cta_kpt<U>(), kCtaWords>(key, n, lo, width, KeyPosition<U>{lo, lz}, mult,
-                                                                              k0, k1, sh.bin, []() {});
+    U lo, hi;
+    block_extent<U, kCtaThreads, KPT>(key, n, sh.bin, &lo, &hi);   // (its barrier also ends the clearing)
+    const unsigned long long width = (unsigned long long)(U)(hi - lo);
+    const U* r;
+    auto none = []() {};
+    if constexpr (MO::is_float) {
+        const auto pos = block_value_position<U, kCtaThreads, KPT>(key, n, out, out.descending(), sh.value);
+        r = n <= kCtaFewKeys
+                ? block_bin_sort<U, kCtaThreads, KPT, kCtaFewWords>(key, n, lo, width, pos,
+                                                                    4u * kCtaFewWords * kCtaThreads, k0, k1, sh.bin, none)
+                : block_bin_sort<U, kCtaThreads, KPT, kCtaWords>(key, n, lo, width, pos, 4u * kCtaWords * kCtaThreads, k0,
+                                                                 k1, sh.bin, none);
+    } else {
+        int lz;
+        uint32_t mult;
+        cut_range_near(width, (uint32_t)(4 * (n <= kCtaFewKeys ? kCtaFewWords : kCtaWords) * kCtaThreads), &lz, &mult);
+        const KeyPosition<U> pos{lo, lz};
+        r = n <= kCtaFewKeys
+                ? block_bin_sort<U, kCtaThreads, KPT, kCtaFewWords>(key, n, lo, width, pos, mult, k0, k1, sh.bin, none)
+                : block_bin_sort<U, kCtaThreads, KPT, kCtaWords>(key, n, lo, width, pos, mult, k0, k1, sh.bin, none);
     }
     for (int i = threadIdx.x; i < n; i += kCtaThreads) store(i, r[i]);
     __syncthreads();
@@ -258,6 +250,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
 
     // ---- range of the keys, from a sample
     U lo, hi;
+    float low = 0.f, scale = 0.f;   // floats: the cut of the sampled values
     {
         U k[8];
         const uint32_t stride = len / (8 * kCtaThreads);
@@ -266,6 +259,11 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
         for (int i = 0; i < 8; ++i)
             if (i * kCtaThreads + tid < m) k[i] = in(src[(uint32_t)(i * kCtaThreads + tid) * (stride ? stride : 1u)]);
         block_extent<U, kCtaThreads, 8>(k, m, sh.bin, &lo, &hi);
+        if constexpr (MO::is_float) {
+            const auto pos = block_value_position<U, kCtaThreads, 8>(k, m, out, out.descending(), sh.value);
+            low = pos.low;
+            scale = pos.scale;
+        }
     }
     const unsigned long long width = (unsigned long long)(U)(hi - lo);
     if (width == 0) {   // one value, as far as the sample shows
@@ -282,12 +280,23 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
     if (want > (uint32_t)kCtaParts) want = (uint32_t)kCtaParts;
     int lz;
     uint32_t mult;
-    const uint32_t np = cut_range(width, want, &lz, &mult);
-    const bool one_value = width < (unsigned long long)np;
+    uint32_t np = cut_range(width, want, &lz, &mult);
+    bool one_value = width < (unsigned long long)np;
+    if (MO::is_float) {
+        np = want;
+        one_value = false;
+    }
     // keys outside the sampled range go to the first and the last part
     auto part_of = [&](U k) {
-        const U d = (k > lo ? k : lo) - lo;
-        return __umulhi(norm32(d < (U)width ? d : (U)width, lz), mult);
+        if constexpr (MO::is_float) {
+            ValuePosition<U, MO> pos(out, 0.f, 0.f, out.descending());
+            pos.low = low;
+            pos.scale = scale;
+            return __umulhi(pos(k), np);
+        } else {
+            const U d = (k > lo ? k : lo) - lo;
+            return __umulhi(norm32(d < (U)width ? d : (U)width, lz), mult);
+        }
     };
 
     // ---- count
@@ -437,10 +446,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
 #pragma unroll
             for (int i = 0; i < KPT; ++i)
                 key[i] = (uint32_t)(i * kCtaThreads + tid) < n ? part[s + (uint32_t)(i * kCtaThreads + tid)] : (U)0;
-            U a, b;
-            block_extent<U, kCtaThreads, KPT>(key, (int)n, sh.bin, &a, &b);
-            cta_local_sort<U>(key, (int)n, a, (unsigned long long)(U)(b - a), smem, sh,
-                              [&](int i, U k) { fin[s + (uint32_t)i] = out(k); });
+            cta_local_sort<U>(key, (int)n, out, smem, sh, [&](int i, U k) { fin[s + (uint32_t)i] = out(k); });
         } else {
             __syncthreads();
         }

@@ -1050,7 +1050,7 @@ __global__ void __launch_bounds__(kHybThreads, 2) hybrid_local(HybArgs a) {
         if (len > (uint32_t)hyb_cap<U>()) {
             __syncthreads();
             U* const at = out + q.start;
-            cta_split_again<U>(at, (U*)a.tmp + q.start, at, len, FloatOut<U>(map), smem, s_cta);
+            cta_split_again<U>(at, (U*)a.tmp + q.start, at, len, GeneralOut<U>(map), smem, s_cta);
             bin_zero<kHybThreads, kHybLocalWords>(k1);
             __syncthreads();
             load(s_q[cur ^ 1]);

@@ -137,9 +137,7 @@ __device__ __forceinline__ void block_tier(const SegArgs& a, unsigned char* smem
 #pragma unroll
     for (int i = 0; i < cta_kpt<U>(); ++i)
         if (i * kSB + (int)threadIdx.x < len) k[i] = in(keys[i * kSB + threadIdx.x]);
-    U mn, mx;
-    block_extent<U, kSB, cta_kpt<U>()>(k, len, sh.bin, &mn, &mx);
-    cta_local_sort<U>(k, len, mn, (unsigned long long)(U)(mx - mn), smem, sh, [&](int i, U x) { keys[i] = out(x); });
+    cta_local_sort<U>(k, len, out, smem, sh, [&](int i, U x) { keys[i] = out(x); });
 }
 
 template <typename U, typename MI, typename MO>

@@ -16,7 +16,6 @@
 // The merge sort had six to nine rounds, each a binary search and a serial
 // merge per thread; the bins have one scan.  Device time of one sort, from a
 // replayed graph: see kSmallRun below for the merge sort's.
-#include <cfloat>
 #include <type_traits>
 
 #include "evosort.h"
@@ -32,37 +31,6 @@ constexpr int kSmallThreads = 512;
 static_assert(kSmallMax <= 16 * kSmallThreads, "largest compiled shape");
 __host__ __device__ constexpr size_t small_up(size_t x) { return (x + 15) / 16 * 16; }
 constexpr int kSmallRun = 16;   // longest insertion-sorted base run
-
-// Position of a float key by its value: (value - smallest) * scale.  Floats of
-// an even spread crowd into the few bit patterns of the largest exponents, so
-// equal stretches of the mapped keys would leave most bins empty; equal
-// stretches of the values do not.  Rounding keeps the order: subtraction,
-// multiplication and the narrowing of doubles never turn two values around.
-// NaNs, which have no value, go to their end of the order, infinities clamp.
-template <typename U>
-__device__ __forceinline__ float key_value(U k, const KeyMap& map);
-template <>
-__device__ __forceinline__ float key_value<uint32_t>(uint32_t k, const KeyMap& map) {
-    return __uint_as_float(map_inv(k, map));
-}
-template <>
-__device__ __forceinline__ float key_value<uint64_t>(uint64_t k, const KeyMap& map) {
-    return __double2float_rn(__longlong_as_double((long long)map_inv(k, map)));
-}
-template <typename U>
-struct ValuePosition {
-    static constexpr bool linear = false;
-    KeyMap map;
-    float low, scale;   // of half the value, so that the widest range stays finite
-    bool descending;
-    __device__ __forceinline__ uint32_t operator()(U k) const {
-        const float f = key_value<U>(k, map);
-        if (f != f) return descending ? 0u : 0xFFFFFFFFu;
-        const float h = 0.5f * f;
-        const float x = (descending ? low - h : h - low) * scale;
-        return x <= 0.f ? 0u : (x >= 4294967040.f ? 0xFFFFFFFFu : (uint32_t)x);
-    }
-};
 
 // KPT keys per thread at most, WPT words of four bins per thread.
 template <typename U, bool PAIRS, bool FLT, int KPT, int WPT>
@@ -104,38 +72,9 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
         return;
     }
     if (FLT) {
-        // smallest and largest finite value, then the same bins by value
+        // the same bins by value
         __shared__ float s_f[2][NT / 32];
-        float a = INFINITY, b = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < KPT; ++i) {
-            if (i * NT + tid < n) {
-                const float f = key_value<U>(key[i], map);
-                if (fabsf(f) < INFINITY) {
-                    a = fminf(a, f);
-                    b = fmaxf(b, f);
-                }
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a = fminf(a, __shfl_xor_sync(0xffffffffu, a, o));
-            b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
-        }
-        if ((tid & 31) == 0) {
-            s_f[0][tid >> 5] = a;
-            s_f[1][tid >> 5] = b;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < NT / 32; ++w) {
-            a = fminf(a, s_f[0][w]);
-            b = fmaxf(b, s_f[1][w]);
-        }
-        const bool desc = map.x != 0;
-        const float range = 0.5f * b - 0.5f * a;   // negative or NaN if no value is finite: one bin
-        const float scale = range > 0.f ? fminf(4294967040.f / range, FLT_MAX) : 0.f;
-        const ValuePosition<U> pos{map, 0.5f * (desc ? b : a), scale, desc};
+        const auto pos = block_value_position<U, NT, KPT>(key, n, GeneralOut<U>(map), map.x != 0, s_f);
         ks = block_bin_sort<U, NT, KPT, WPT, PAIRS, true>(key, n, lo, width, pos, (uint32_t)(4 * WPT * NT), k0, k1, sh,
                                                           []() {}, x0);
     } else {
@@ -156,12 +95,36 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
         for (int i = 0; i < KPT; ++i)
             if (i * NT + tid < n) k0[i * NT + tid] = key[i];
         __syncthreads();
-        const int passes = (64 - __clzll((long long)width) + 7) / 8;
-        int rounds = 1;
-        while ((kSmallRun << rounds) < n) ++rounds;
-        const int which = passes <= rounds
-                              ? smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, passes, counts, sh.wsum)
-                              : smem_merge_sort<U, PAIRS, kSmallRun>(k0, k1, v0, v1, n, tins);
+        const int bits = 64 - __clzll((long long)width), passes = (bits + 7) / 8;
+        // Over a wide range two passes over the leading 16 bits may do: a few
+        // frequent values rarely share these.  Tried if the first keys of each
+        // warp share them only with equal keys; one look at the neighbours
+        // shows whether the keys are in order (16 values, 3,000 int64 keys:
+        // 27 us by eight passes, 11 so).
+        bool lead = false, sorted = false;
+        if (passes > 3) {
+            bool other = false;
+            const uint32_t m = __ballot_sync(0xffffffffu, tid < n);
+            if (tid < n) {
+                const uint32_t peers = __match_any_sync(m, digit_of((U)(key[0] - lo), bits - 16, 0xFFFFu));
+                other = k0[tid / 32 * 32 + __ffs((int)peers) - 1] != key[0];
+            }
+            lead = !__syncthreads_or(other);
+        }
+        int which = 0;
+        if (lead) {
+            smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, bits - 16, 2, counts, sh.wsum);   // back in k0
+            bool down = false;
+            for (int i = tid + 1; i < n; i += NT) down |= k0[i] < k0[i - 1];
+            sorted = !__syncthreads_or(down);
+        }
+        if (!sorted) {   // (equal keys are still in input order)
+            int rounds = 1;
+            while ((kSmallRun << rounds) < n) ++rounds;
+            which = passes <= rounds
+                        ? smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, 0, passes, counts, sh.wsum)
+                        : smem_merge_sort<U, PAIRS, kSmallRun>(k0, k1, v0, v1, n, tins);
+        }
         ks = which ? k1 : k0;
         vs = which ? v1 : v0;
         by_position = false;

@@ -161,13 +161,13 @@ __device__ int smem_merge_sort(U* k0, U* k1, uint32_t* v0, uint32_t* v1, int len
 // ---------------------------------------------------------------------------
 // CTA radix sort (Algorithms 4a/4b in one CTA): stable LSD passes over 8-bit
 // digits of k - lo, from k0/v0 through k1/v1, for len <= 32 * COLS keys per
-// warp.  passes: digits of the keys' range.  counts: NT / 32 x 256 16-bit
+// warp.  passes: digits, from bit first on.  counts: NT / 32 x 256 16-bit
 // counters.  Returns 0 if the result is in k0/v0, 1 if in k1/v1.  All threads
 // of the CTA must call it.
 // ---------------------------------------------------------------------------
 template <typename U, bool PAIRS, int NT, int COLS>
-__device__ __noinline__ int smem_radix_sort(U* k0, U* k1, uint32_t* v0, uint32_t* v1, int len, U lo, int passes,
-                                            uint16_t* counts, uint32_t* scratch) {
+__device__ __noinline__ int smem_radix_sort(U* k0, U* k1, uint32_t* v0, uint32_t* v1, int len, U lo, int first,
+                                            int passes, uint16_t* counts, uint32_t* scratch) {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cols = (len + NT - 1) / NT;   // columns of 32 keys per warp, consecutive in the array
@@ -187,7 +187,7 @@ __device__ __noinline__ int smem_radix_sort(U* k0, U* k1, uint32_t* v0, uint32_t
                 const bool have = s < len;
                 key[i] = have ? k0[s] : (U)0;
                 if (PAIRS) val[PAIRS ? i : 0] = have ? v0[s] : 0u;
-                const uint32_t d = digit_of((U)(key[i] - lo), 8 * p, 0xFFu);
+                const uint32_t d = digit_of((U)(key[i] - lo), first + 8 * p, 0xFFu);
                 uint32_t peers = __ballot_sync(0xffffffffu, have);   // lanes with the same digit
 #pragma unroll
                 for (int b = 0; b < 8; ++b) {

@@ -69,3 +69,27 @@ def test_segments_of_every_shape(evo, dtype, kind):
     evo.segmented_sort(k, offs.cuda())
     evo.sync()
     assert np.array_equal(bits(k), bits(want))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64], ids=["float32", "float64"])
+@pytest.mark.parametrize("kind", ["normal", "specials", "orders", "infinite"])
+def test_float_segments_cut_by_value(evo, dtype, kind):
+    """Float keys are cut by their values: infinities, NaNs and zeros of both
+    signs, values whose range is not finite, and ranges that values cut badly."""
+    lengths = np.array([0, 1, 255, 257, 1536, 1537, 6144, 6145, 8192, 8193, 50_001, 300_007])
+    offs = np.concatenate([[0], np.cumsum(lengths)]).astype(np.uint64)
+    r = np.random.default_rng(11)
+    n = int(offs[-1])
+    x = r.normal(0, 1, n)
+    if kind == "orders":
+        x = np.ldexp(x, r.integers(-100, 100, n))
+    elif kind == "specials":
+        x = np.choose(r.integers(0, 12, n), [x * np.finfo(dtype).max / 16, np.inf, -np.inf, np.nan, -np.nan, 0.0, -0.0] + [x] * 5)
+    elif kind == "infinite":
+        x = np.where(r.random(n) < 0.5, np.inf, -np.inf)
+    x = x.astype(dtype)
+    want = oracle.segmented_sort(x, offs)
+    k = torch.from_numpy(x.copy()).cuda()
+    evo.segmented_sort(k, torch.from_numpy(offs.astype(np.int64)).cuda())
+    evo.sync()
+    assert np.array_equal(bits(k), bits(want))

@@ -34,6 +34,7 @@ def ints(kind, n, dtype):
             "few": lambda: r.integers(0, 5, n).astype(dtype), "equal": lambda: np.full(n, -7, dtype),
             "pairs": lambda: (r.integers(0, n, n) // 2).astype(dtype),
             "clump": lambda: np.where(r.random(n) < 0.5, r.integers(0, 40, n), r.integers(lo // 2, hi // 2, n)).astype(dtype),
+            "late": lambda: np.where((np.arange(n) < 512) | (r.random(n) < 0.5), hi, r.integers(lo, lo + 99, n)).astype(dtype),
             "ends": lambda: np.where(r.random(n) < 0.5, lo, hi).astype(dtype)}[kind]()
 
 
@@ -47,7 +48,6 @@ def floats(kind, n, dtype):
          "close": lambda: 1.0 + r.integers(0, 3 * n, n) * float(info.eps), "infinite": lambda: np.full(n, np.inf)}[kind]()
     x = x.astype(dtype)
     if kind in ("specials", "infinite"):
-        neg_nan = np.array([-np.nan], dtype)
         neg_nan = np.copysign(np.array([np.nan], dtype), dtype(-1))
         pick = r.integers(0, 12, n)
         for i, v in enumerate((np.inf, -np.inf, np.nan, -0.0, 0.0)):
@@ -86,7 +86,7 @@ def check(evo, a):
 
 
 @pytest.mark.parametrize("dtype", [np.int32, np.int64], ids=["int32", "int64"])
-@pytest.mark.parametrize("kind", ["spread", "few", "equal", "pairs", "clump", "ends"])
+@pytest.mark.parametrize("kind", ["spread", "few", "equal", "pairs", "clump", "ends", "late"])
 def test_integers(evo, dtype, kind):
     for n in SIZES:
         check(evo, ints(kind, n, dtype))
