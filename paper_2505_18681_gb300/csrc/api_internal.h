@@ -69,8 +69,6 @@ struct SampleInfo {
     int order = 0;
     bool spread = false;   // worth trying the partition sort on
 };
-int classify_sample(const unsigned char* buf, size_t m, int dt, bool descending = false,
-                    SampleInfo* info = nullptr);
 int classify_host(const void* keys, size_t n, int dt, bool descending = false);
 // evosort_plan for a sort in the given direction (the class is read in the
 // order the sort will produce)

@@ -5,6 +5,7 @@
 // GA run per size); the class adds what the data itself changes on a GPU:
 // which digits are constant, how many lanes of a warp share a digit.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -46,69 +47,263 @@ uint64_t host_map(uint64_t u, int dt, bool descending) {
 
 }  // namespace
 
-// Class of a sample of m keys (raw bytes, m x key width), taken at stride
-// n / m from an array of n keys, read in the order of the sort's direction.
-// With info, the distinct sampled keys (mapped, ascending) when there are at
-// most kDictMax of them, and the sample's order (1: no pair falls, -1: no
-// pair rises, 0: both happen).
-int classify_sample(const unsigned char* buf, size_t m, int dt, bool descending, SampleInfo* info) {
+// What the dispatcher reads off a sample of mapped keys.
+struct SampleStats {
+    uint64_t vary, least, most;   // bits that vary; smallest and largest key
+    // strict rises and falls between neighbours: equal neighbours say nothing
+    // about order (90% zeros would otherwise read as both sorted and reverse
+    // sorted)
+    uint32_t up, down;
+    // runs of equal keys once sorted: their number, the longest, the keys in
+    // runs of four or more
+    uint32_t distinct, longest, often;
+    uint32_t topmax;              // keys that share the most common top byte
+    uint64_t dict[kDictMax];      // the distinct keys, ascending, if distinct <= kDictMax
+};
+
+// Class of the sample of m keys.  With info, the distinct sampled keys when
+// there are at most kDictMax of them, and the sample's order (1: no pair falls,
+// -1: no pair rises, 0: both happen).
+static int class_of(const SampleStats& q, size_t m, int dt, SampleInfo* info) {
     const int w = dtype_bytes(dt);
-    std::vector<uint64_t> raw(m, 0);
-    for (size_t i = 0; i < m; ++i) {
-        uint64_t u = 0;
-        std::memcpy(&u, buf + i * w, w);
-        raw[i] = host_map(u, dt, descending);
-    }
-    // strict rises and falls between neighbours: equal neighbours say
-    // nothing about order (90% zeros would otherwise read as both sorted and
-    // reverse sorted)
-    size_t up = 0, down = 0;
-    uint64_t vary = 0;
-    for (size_t i = 0; i + 1 < m; ++i) {
-        up += raw[i] < raw[i + 1];
-        down += raw[i] > raw[i + 1];
-    }
-    for (size_t i = 0; i < m; ++i) vary |= raw[i] ^ raw[0];
-    std::vector<uint64_t> sorted(raw);
-    std::sort(sorted.begin(), sorted.end());
-    // runs of equal keys: their number (the first kDictMax + 1 values are kept
-    // at the front), the longest, and the keys in runs of four or more
-    const uint64_t least = sorted.front(), most = sorted.back();
-    size_t distinct = 0, longest = 0, often = 0;
-    for (size_t i = 0; i < m;) {
-        const uint64_t v = sorted[i];
-        size_t j = i + 1;
-        while (j < m && sorted[j] == v) ++j;
-        if (distinct <= (size_t)kDictMax) sorted[distinct] = v;   // distinct <= i
-        ++distinct;
-        longest = std::max(longest, j - i);
-        if (j - i >= 4) often += j - i;
-        i = j;
-    }
     if (info) {
         info->dict.clear();
-        if (distinct <= (size_t)kDictMax) info->dict.assign(sorted.begin(), sorted.begin() + distinct);
-        info->order = down == 0 ? 1 : (up == 0 ? -1 : 0);
+        if (q.distinct <= (uint32_t)kDictMax) info->dict.assign(q.dict, q.dict + q.distinct);
+        info->order = q.down == 0 ? 1 : (q.up == 0 ? -1 : 0);
         // (the path's own sample decides in the end; this one only spares the
         // launches and the wait where it is sure to say no)
-        const bool wide = ((most - least) >> 24) != 0;
-        info->spread = longest * 4 <= m && (wide ? longest * 128 <= m : often * 4 >= m);
+        const bool wide = ((q.most - q.least) >> 24) != 0;
+        info->spread = (size_t)q.longest * 4 <= m && (wide ? (size_t)q.longest * 128 <= m : (size_t)q.often * 4 >= m);
     }
-    // top-byte concentration: share of the sample in the most common top byte
-    size_t top[256] = {0};
-    for (size_t i = 0; i < m; ++i) top[(raw[i] >> (8 * w - 8)) & 0xFF] += 1;
-    const size_t topmax = *std::max_element(top, top + 256);
     int bits = 0;
-    while (bits < 64 && (vary >> bits)) ++bits;
-    if (distinct == 1) return EVOSORT_CLASS_CONSTANT;
-    if (distinct <= 64) return EVOSORT_CLASS_FEW;          // few values, whatever their order
-    const size_t moves = up + down;
-    if (up >= 0.9 * (double)moves) return EVOSORT_CLASS_SORTED;
-    if (down >= 0.9 * (double)moves) return EVOSORT_CLASS_REVERSE;
+    while (bits < 64 && (q.vary >> bits)) ++bits;
+    if (q.distinct == 1) return EVOSORT_CLASS_CONSTANT;
+    if (q.distinct <= 64) return EVOSORT_CLASS_FEW;          // few values, whatever their order
+    const uint32_t moves = q.up + q.down;
+    if (q.up >= 0.9 * (double)moves) return EVOSORT_CLASS_SORTED;
+    if (q.down >= 0.9 * (double)moves) return EVOSORT_CLASS_REVERSE;
     if (bits <= 16) return EVOSORT_CLASS_NARROW16;
     if (bits <= 4 * w) return EVOSORT_CLASS_NARROW;          // at most half the key bits vary
-    if (topmax * 4 > m) return EVOSORT_CLASS_SKEWED;         // a quarter in one top byte
+    if ((size_t)q.topmax * 4 > m) return EVOSORT_CLASS_SKEWED;   // a quarter in one top byte
     return EVOSORT_CLASS_RANDOM;
+}
+
+// ---------------------------------------------------------------------------
+// K_s: the statistics of a device array's sample, by one CTA: keys i * stride,
+// i < m <= kSample, of n.  Equal keys meet in a hash table (twice as many
+// slots as keys, linear probing), so that no sort is needed: a slot holds the
+// first such key's place + 1, and their number << 16.  The keys of a warp are
+// grouped before the table and the byte counts see them, so that frequent
+// values do not queue up.  Bound by the latency of the strided reads and of
+// its barriers.  It stands in place of a strided copy of the keys to the host
+// and a sort there, which cost 30 to 90 us of every call with a table, the most
+// on keys that differ much: 300,000 uniform int64 keys 306 -> 154 us (the sort
+// included), sorted ones 94 -> 74 us; 9e6 reversed ones 115 -> 109.
+// ---------------------------------------------------------------------------
+constexpr int kSampleThreads = 1024;
+constexpr int kSampleSlots = 2 * kSample;
+constexpr int kStatsSlots = 64;   // calls that sample at the same time
+__device__ SampleStats g_stats[kStatsSlots];
+
+__device__ __forceinline__ uint32_t sample_hash(uint64_t k) {
+    k ^= k >> 32;   // (the multipliers of splitmix64)
+    k *= 0xbf58476d1ce4e5b9ull;
+    k ^= k >> 27;
+    k *= 0x94d049bb133111ebull;
+    return (uint32_t)(k >> 40) & (uint32_t)(kSampleSlots - 1);
+}
+
+template <typename U>
+__device__ __forceinline__ U load_any(const unsigned char* p, bool aligned) {
+    if (aligned) return *(const U*)p;
+    U x = 0;
+    for (int b = 0; b < (int)sizeof(U); ++b) x |= (U)p[b] << (8 * b);
+    return x;
+}
+
+template <typename U>
+__global__ void __launch_bounds__(kSampleThreads) sample_stats(const unsigned char* keys, size_t stride, int m,
+                                                               KeyMap map, SampleStats* to, int slot) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    U* s_key = (U*)smem;                              // kSample
+    uint32_t* s_slot = (uint32_t*)(s_key + kSample);  // kSampleSlots
+    __shared__ uint32_t s_top[256];
+    __shared__ uint32_t s_up, s_down, s_distinct, s_longest, s_often, s_ndict, s_topmax;
+    __shared__ unsigned long long s_vary, s_least, s_most;
+    __shared__ U s_dict[kDictMax];
+    constexpr int PER = kSample / kSampleThreads;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool aligned = (uintptr_t)keys % sizeof(U) == 0;
+    U k[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = j * kSampleThreads + tid;
+        if (i < m) k[j] = load_any<U>(keys + (size_t)i * stride * sizeof(U), aligned);
+    }
+    for (int i = tid; i < kSampleSlots; i += kSampleThreads) s_slot[i] = 0u;
+    if (tid < 256) s_top[tid] = 0u;
+    if (tid == 0) {
+        s_up = s_down = s_distinct = s_longest = s_often = s_ndict = s_topmax = 0u;
+        s_vary = s_most = 0ull;
+        s_least = ~0ull;
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = j * kSampleThreads + tid;
+        if (i < m) s_key[i] = k[j] = map_fwd(k[j], map);
+    }
+    __syncthreads();
+    // ---- order, range, varying bits, top bytes, equal keys
+    uint32_t up = 0, down = 0;
+    unsigned long long vary = 0, least = ~0ull, most = 0;
+    const U first = s_key[0];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = j * kSampleThreads + tid;
+        const uint32_t here = __ballot_sync(0xffffffffu, i < m);
+        if (i < m) {
+            const U x = k[j];
+            if (i + 1 < m) {
+                up += x < s_key[i + 1];
+                down += x > s_key[i + 1];
+            }
+            vary |= (unsigned long long)(U)(x ^ first);
+            least = min(least, (unsigned long long)x);
+            most = max(most, (unsigned long long)x);
+            const uint32_t top = (uint32_t)(x >> (8 * sizeof(U) - 8));
+            const uint32_t tp = __match_any_sync(here, top);
+            if (lane == __ffs((int)tp) - 1) atomicAdd(&s_top[top], (uint32_t)__popc(tp));
+            const uint32_t kp = __match_any_sync(here, x);
+            if (lane == __ffs((int)kp) - 1) {
+                const uint32_t count = (uint32_t)__popc(kp) << 16;
+                uint32_t h = sample_hash((uint64_t)x);
+                for (int probe = 0; probe < kSampleSlots; ++probe) {   // (ends: more slots than keys)
+                    const uint32_t old = atomicCAS(&s_slot[h], 0u, count | (uint32_t)(i + 1));
+                    if (old == 0u) break;
+                    if (s_key[(old & 0xFFFFu) - 1u] == x) {
+                        atomicAdd(&s_slot[h], count);
+                        break;
+                    }
+                    h = (h + 1u) & (uint32_t)(kSampleSlots - 1);
+                }
+            }
+        }
+    }
+    up = __reduce_add_sync(0xffffffffu, up);
+    down = __reduce_add_sync(0xffffffffu, down);
+    const uint32_t vlo = __reduce_or_sync(0xffffffffu, (uint32_t)vary);
+    const uint32_t vhi = __reduce_or_sync(0xffffffffu, (uint32_t)(vary >> 32));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        least = min(least, __shfl_xor_sync(0xffffffffu, least, o));
+        most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    }
+    if (lane == 0) {
+        atomicAdd(&s_up, up);
+        atomicAdd(&s_down, down);
+        atomicOr(&s_vary, (unsigned long long)vhi << 32 | vlo);
+        atomicMin(&s_least, least);
+        atomicMax(&s_most, most);
+    }
+    __syncthreads();
+    // ---- runs
+    uint32_t distinct = 0, longest = 0, often = 0;
+    for (int i = tid; i < kSampleSlots; i += kSampleThreads) {
+        const uint32_t c = s_slot[i] >> 16;
+        distinct += c != 0u;
+        longest = max(longest, c);
+        if (c >= 4u) often += c;
+    }
+    distinct = __reduce_add_sync(0xffffffffu, distinct);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    often = __reduce_add_sync(0xffffffffu, often);
+    const uint32_t top = __reduce_max_sync(0xffffffffu, tid < 256 ? s_top[tid] : 0u);
+    if (lane == 0) {
+        atomicAdd(&s_distinct, distinct);
+        atomicMax(&s_longest, longest);
+        atomicAdd(&s_often, often);
+        atomicMax(&s_topmax, top);
+    }
+    __syncthreads();
+    SampleStats* const q = to ? to : g_stats + slot;
+    const uint32_t nd = s_distinct;
+    if (nd <= (uint32_t)kDictMax) {   // the distinct keys, each to its rank
+        for (int i = tid; i < kSampleSlots; i += kSampleThreads) {
+            const uint32_t f = s_slot[i] & 0xFFFFu;
+            if (f) s_dict[atomicAdd(&s_ndict, 1u)] = s_key[f - 1u];   // (nd of them)
+        }
+        __syncthreads();
+        if (tid < (int)nd) {
+            const U x = s_dict[tid];
+            uint32_t rank = 0;
+            for (uint32_t i = 0; i < nd; ++i) rank += s_dict[i] < x;
+            q->dict[rank] = (uint64_t)x;
+        }
+    }
+    if (tid == 0) {
+        q->vary = s_vary;
+        q->least = s_least;
+        q->most = s_most;
+        q->up = s_up;
+        q->down = s_down;
+        q->distinct = nd;
+        q->longest = s_longest;
+        q->often = s_often;
+        q->topmax = s_topmax;
+    }
+}
+
+template <typename U>
+static cudaError_t launch_sample(const void* keys, size_t stride, size_t m, KeyMap map, SampleStats* to, int slot,
+                                 cudaStream_t s) {
+    constexpr int bytes = kSample * (int)sizeof(U) + kSampleSlots * 4;
+    static_assert(bytes + 2048 <= 64 * 1024 + 4096, "two CTAs per SM and a little more");
+    const cudaError_t e =
+        cudaFuncSetAttribute(sample_stats<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    sample_stats<U><<<1, kSampleThreads, bytes, s>>>((const unsigned char*)keys, stride, (int)m, map, to, slot);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+// The statistics of keys i * stride, i < m, of a device array, read back
+// (synchronises the stream).  They pass through one of a fixed set of places
+// in device memory; a call that finds all of them taken allocates its own.
+static cudaError_t sample_device(const void* keys, size_t stride, size_t m, int dt, bool descending, SampleStats* q,
+                                 cudaStream_t s) {
+    // memory that the GPU cannot read is refused here, before a kernel meets it
+    cudaPointerAttributes at{};
+    cudaError_t e = cudaPointerGetAttributes(&at, keys);
+    if (e == cudaSuccess && at.type == cudaMemoryTypeUnregistered) {
+        int dev = 0, pageable = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev);
+        if (e == cudaSuccess && !pageable) e = cudaErrorInvalidValue;
+    }
+    if (e != cudaSuccess) return e;
+    static std::atomic<uint64_t> taken{0};
+    static_assert(kStatsSlots == 64, "one bit each");
+    int slot = -1;
+    uint64_t t = taken.load();
+    while (slot < 0 && ~t) {
+        int free = 0;
+        while ((t >> free) & 1) ++free;
+        if (taken.compare_exchange_weak(t, t | 1ull << free)) slot = free;
+    }
+    SampleStats* own = nullptr;
+    e = slot < 0 ? cudaMallocAsync((void**)&own, sizeof(SampleStats), s) : cudaSuccess;
+    const KeyMap map = key_map_for(dt, descending);
+    if (e == cudaSuccess)
+        e = dtype_bytes(dt) == 4 ? launch_sample<uint32_t>(keys, stride, m, map, own, slot, s)
+                                 : launch_sample<uint64_t>(keys, stride, m, map, own, slot, s);
+    if (e == cudaSuccess)
+        e = own ? cudaMemcpyAsync(q, own, sizeof(*q), cudaMemcpyDeviceToHost, s)
+                : cudaMemcpyFromSymbolAsync(q, g_stats, sizeof(*q), (size_t)slot * sizeof(*q), cudaMemcpyDeviceToHost, s);
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = es;
+    if (own) cudaFreeAsync(own, s);
+    if (slot >= 0) taken.fetch_and(~(1ull << slot));
+    return e;
 }
 
 // Class of n keys in host memory, from the same strided sample the device
@@ -118,9 +313,36 @@ int classify_host(const void* keys, size_t n, int dt, bool descending) {
     const int w = dtype_bytes(dt);
     const size_t m = n < (size_t)kSample ? n : (size_t)kSample;
     const size_t stride = n / m;
-    std::vector<unsigned char> buf(m * w);
-    for (size_t i = 0; i < m; ++i) std::memcpy(buf.data() + i * w, (const unsigned char*)keys + i * stride * w, w);
-    return classify_sample(buf.data(), m, dt, descending);
+    std::vector<uint64_t> raw(m, 0);
+    for (size_t i = 0; i < m; ++i) {
+        uint64_t u = 0;
+        std::memcpy(&u, (const unsigned char*)keys + i * stride * w, w);
+        raw[i] = host_map(u, dt, descending);
+    }
+    SampleStats q{};
+    for (size_t i = 0; i + 1 < m; ++i) {
+        q.up += raw[i] < raw[i + 1];
+        q.down += raw[i] > raw[i + 1];
+    }
+    uint32_t top[256] = {0};
+    for (size_t i = 0; i < m; ++i) {
+        q.vary |= raw[i] ^ raw[0];
+        top[(raw[i] >> (8 * w - 8)) & 0xFF] += 1;
+    }
+    q.topmax = *std::max_element(top, top + 256);
+    std::sort(raw.begin(), raw.end());
+    q.least = raw.front();
+    q.most = raw.back();
+    for (size_t i = 0; i < m;) {
+        size_t j = i + 1;
+        while (j < m && raw[j] == raw[i]) ++j;
+        if (q.distinct < (uint32_t)kDictMax) q.dict[q.distinct] = raw[i];
+        ++q.distinct;
+        q.longest = std::max(q.longest, (uint32_t)(j - i));
+        if (j - i >= 4) q.often += (uint32_t)(j - i);
+        i = j;
+    }
+    return class_of(q, m, dt, nullptr);
 }
 
 // Table entry for (dt, n, cls): the class itself at the nearest size bucket,
@@ -165,23 +387,18 @@ evosort_status classify_device(const void* keys, size_t n, int dt, void* stream,
         set_error("evosort_classify: bad argument");
         return EVOSORT_ERR_INVALID;
     }
-    const int w = dtype_bytes(dt);
     if (n < 2) {
         *cls = EVOSORT_CLASS_CONSTANT;
         return EVOSORT_OK;
     }
     const size_t m = n < (size_t)kSample ? n : (size_t)kSample;
-    const size_t stride = n / m;
-    std::vector<unsigned char> buf(m * w);
-    // one strided device-to-host copy of m keys
-    cudaError_t e = cudaMemcpy2DAsync(buf.data(), w, keys, stride * w, w, m, cudaMemcpyDeviceToHost,
-                                      (cudaStream_t)stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
+    SampleStats q;
+    const cudaError_t e = sample_device(keys, n / m, m, dt, descending, &q, (cudaStream_t)stream);
     if (e != cudaSuccess) {
-        set_error(std::string("evosort_classify: sample copy: ") + cudaGetErrorString(e));
+        set_error(std::string("evosort_classify: sample: ") + cudaGetErrorString(e));
         return EVOSORT_ERR_CUDA;
     }
-    *cls = classify_sample(buf.data(), m, dt, descending, info);
+    *cls = class_of(q, m, dt, info);
     return EVOSORT_OK;
 }
 
