@@ -696,7 +696,8 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
         // spread keys: the partition sort (an array of few values or in order
         // has been sorted above, or proved to be neither)
         fused = true;   // (the table's tile is for the chain of launches)
-        hybrid = n >= kHybridMinSync && info.order == 0 && info.spread ? HYBRID_SYNC : HYBRID_OFF;
+        hybrid = n >= (info.wide ? kHybridMinSync : kHybridMinNarrow) && info.order == 0 && info.spread ? HYBRID_SYNC
+                                                                                                    : HYBRID_OFF;
         if (p) {
             planned.stream = p->stream;
             planned.workspace = p->workspace;

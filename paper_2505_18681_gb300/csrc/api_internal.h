@@ -68,6 +68,7 @@ struct SampleInfo {
     std::vector<uint64_t> dict;
     int order = 0;
     bool spread = false;   // worth trying the partition sort on
+    bool wide = false;     // more than 24 bits
 };
 int classify_host(const void* keys, size_t n, int dt, bool descending = false);
 // evosort_plan for a sort in the given direction (the class is read in the
@@ -123,6 +124,9 @@ constexpr size_t kFusedMin = 2048;
 // verdict, and where the radix kernels are enqueued after it in any case.
 constexpr size_t kHybridMinSync = (size_t)1 << 21;
 constexpr size_t kHybridMinAsync = (size_t)1 << 23;
+// The same for keys that span 24 bits or less, which the radix sort needs three
+// passes at most for.
+constexpr size_t kHybridMinNarrow = (size_t)1 << 26;
 size_t radix_workspace_bytes(size_t n, int w, bool pairs, const Plan& pl);
 int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n, int dt,
                const Plan& pl, void* ws, size_t ws_bytes, cudaStream_t s, std::string* err);

@@ -72,7 +72,7 @@ static int class_of(const SampleStats& q, size_t m, int dt, SampleInfo* info) {
         info->order = q.down == 0 ? 1 : (q.up == 0 ? -1 : 0);
         // (the path's own sample decides in the end; this one only spares the
         // launches and the wait where it is sure to say no)
-        const bool wide = ((q.most - q.least) >> 24) != 0;
+        const bool wide = info->wide = ((q.most - q.least) >> 24) != 0;
         info->spread = (size_t)q.longest * 4 <= m && (wide ? (size_t)q.longest * 128 <= m : (size_t)q.often * 4 >= m);
     }
     int bits = 0;

@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(1024) hybrid_sample(HybArgs a) {
     bool often = false;
     for (int i = tid; i < kHybSample; i += NT) often |= s_hash[i] >= (uint32_t)kHybRepeat;
     if ((__syncthreads_or(often) != 0) == ((span >> 24) != 0)) return;
+    if ((span >> 24) == 0 && a.n < kHybridMinNarrow) return;
 
     // a range that needs the top bit is widened to the whole type, so that the
     // high word of a 64-bit key is its position
