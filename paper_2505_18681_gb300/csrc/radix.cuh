@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kHistThreads) radix_histogram8(RadixArgs a) {
 
 // ---------------------------------------------------------------------------
 // K2: exclusive prefix sum of each pass's digit counts, trivial-pass test and
-// the buffer chain.  One CTA of 1024 threads.
+// the buffer chain.  One CTA of 1024 threads, a warp per pass.
 // ---------------------------------------------------------------------------
 // Adaptive ranking (rank mode 4): a pass ranks with match.any when its digit
 // is concentrated, else with shared match masks.  Concentration is the sum
@@ -424,48 +424,46 @@ __global__ void __launch_bounds__(kHistThreads) radix_histogram8(RadixArgs a) {
 
 static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int inplace) {
     chain_wait();
-    __shared__ unsigned long long s_scr[33];
     __shared__ int s_trivial[64];
     __shared__ int s_conc[64];
-    __shared__ double s_sq[32];
     if (hybrid_done(a.hyb)) return;   // the descriptors stay zero: no pass and no fixup runs
     const int bins = 1 << a.d;
-    const int per = (bins + 1023) / 1024;   // consecutive bins per thread (<= 2)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // a rebased sort (K1b ran) plans from the digit counts of key - min
-    if (a.range && (a.range[RNG_FLAGS] & RNG_REBASED)) {
-        for (int i = threadIdx.x; i < (a.npass << a.d); i += blockDim.x) a.counts[i] = a.counts2[i];
-        __syncthreads();
-    }
-    for (int p = 0; p < a.npass; ++p) {
-        unsigned long long* c = a.counts + (size_t)p * bins;
-        unsigned long long local[2] = {0, 0};
-        unsigned long long sum = 0;
-        int triv = 0;
+    const unsigned long long* const from = a.range && (a.range[RNG_FLAGS] & RNG_REBASED) ? a.counts2 : a.counts;
+    const double nn = (double)a.n * (double)a.n;
+    // a warp per pass, so that the passes' scans run side by side (bound by
+    // their latency: 11 us for 64-bit keys, 41 with one pass after the other)
+    for (int p = warp; p < a.npass; p += 32) {
+        unsigned long long* const c = a.counts + (size_t)p * bins;
+        const unsigned long long* const f = from + (size_t)p * bins;
+        unsigned long long before = 0;
+        bool triv = false;
         double sq = 0.0;
-        for (int j = 0; j < per; ++j) {
-            const int b = threadIdx.x * per + j;
-            local[j] = b < bins ? c[b] : 0ull;
-            if (local[j] == (unsigned long long)a.n) triv = 1;
-            sum += local[j];
-            sq += (double)local[j] * (double)local[j];
+        for (int b0 = 0; b0 < bins; b0 += 256) {
+            unsigned long long v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = b0 + 32 * j + lane < bins ? f[b0 + 32 * j + lane] : 0ull;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                triv |= v[j] == (unsigned long long)a.n;
+                sq += (double)v[j] * (double)v[j];
+                unsigned long long inc = v[j];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                if (b0 + 32 * j + lane < bins) c[b0 + 32 * j + lane] = before + inc - v[j];
+                before += __shfl_sync(0xffffffffu, inc, 31);
+            }
         }
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        if ((threadIdx.x & 31) == 0) s_sq[threadIdx.x >> 5] = sq;
-        const int any_triv = __syncthreads_or(triv);
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < 32; ++w) t += s_sq[w];
-            const double nn = (double)a.n * (double)a.n;
-            s_conc[p] = (t > a.conc_later * nn ? 1 : 0) | (t > a.conc_first * nn ? 2 : 0);
+        triv = __any_sync(0xffffffffu, triv);
+        if (lane == 0) {
+            s_conc[p] = (sq > a.conc_later * nn ? 1 : 0) | (sq > a.conc_first * nn ? 2 : 0);
+            s_trivial[p] = triv;
         }
-        unsigned long long tot;
-        unsigned long long ex = block_exclusive_scan<1024>(sum, s_scr, &tot);
-        for (int j = 0; j < per; ++j) {
-            const int b = threadIdx.x * per + j;
-            if (b < bins) c[b] = ex;
-            ex += local[j];
-        }
-        if (threadIdx.x == 0) s_trivial[p] = any_triv;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
