@@ -93,6 +93,8 @@ _lib = None
 def library():
     """The loaded ctypes handle of libevosort.so (raises if it is not built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_build.LIB):
@@ -201,6 +203,10 @@ def _need_cuda(*ts):
 
 def _stream_handle(stream) -> int:
     if stream is None:
+        # (a small sort takes the GPU 3 us: the checks of is_available and the
+        # Stream object would be a third of the call)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
         if not torch.cuda.is_available():
             return 0   # host-only calls (tables, argument checks): the legacy default stream
         stream = torch.cuda.current_stream()
@@ -213,22 +219,34 @@ def make_params(algo=None, digit_bits=0, keys_per_thread=0, block_size=0, insert
                 rank_mode=0, seg_block_cap=0, stream=None, workspace: torch.Tensor | None = None,
                 descending=False, pass_kernel=0, adapt_later=0, adapt_first=0, seg_warp_cap=0, small_cap=0,
                 seg_giant=0) -> Params:
-    p = Params()
-    library().evosort_default_params(ctypes.byref(p))
-    p.algo = ALGOS[algo]
-    p.digit_bits = int(digit_bits or 0)
-    p.keys_per_thread = int(keys_per_thread or 0)
-    p.block_size = int(block_size or 0)
-    p.insertion_threshold = int(insertion_threshold or 0)
-    p.rank_mode = int(rank_mode or 0)
-    p.seg_block_cap = int(seg_block_cap or 0)
-    p.descending = 1 if descending else 0
-    p.pass_kernel = int(pass_kernel or 0)
-    p.adapt_later = int(adapt_later or 0)
-    p.adapt_first = int(adapt_first or 0)
-    p.seg_warp_cap = int(seg_warp_cap or 0)
-    p.small_cap = int(small_cap or 0)
-    p.seg_giant = int(seg_giant or 0)
+    library()
+    p = Params(ALGOS[algo])   # all else 0: the defaults
+    if digit_bits:
+        p.digit_bits = int(digit_bits)
+    if keys_per_thread:
+        p.keys_per_thread = int(keys_per_thread)
+    if block_size:
+        p.block_size = int(block_size)
+    if insertion_threshold:
+        p.insertion_threshold = int(insertion_threshold)
+    if rank_mode:
+        p.rank_mode = int(rank_mode)
+    if seg_block_cap:
+        p.seg_block_cap = int(seg_block_cap)
+    if pass_kernel:
+        p.pass_kernel = int(pass_kernel)
+    if adapt_later:
+        p.adapt_later = int(adapt_later)
+    if adapt_first:
+        p.adapt_first = int(adapt_first)
+    if seg_warp_cap:
+        p.seg_warp_cap = int(seg_warp_cap)
+    if small_cap:
+        p.small_cap = int(small_cap)
+    if seg_giant:
+        p.seg_giant = int(seg_giant)
+    if descending:
+        p.descending = 1
     p.stream = _stream_handle(stream)
     if workspace is not None:
         p.workspace = workspace.data_ptr()
