@@ -91,7 +91,8 @@ typedef struct {
                                  half of the SMs a tile */
     int insertion_threshold;  /* mergesort base-run length T_insertion, 2..2048
                                  (default 32; Section 4.2 bounds); the one-CTA
-                                 small-array path caps its runs at 16 keys */
+                                 small-array path caps its runs at 16 keys where
+                                 it merges */
     int rank_mode;            /* radix tile ranking (how a warp finds lanes with
                                  equal digits): 1 = match.any (d = 8 only),
                                  2 = one ballot per digit bit (any d),
@@ -105,7 +106,7 @@ typedef struct {
                                      only */
     int seg_block_cap;        /* segmented sort: segments up to this many keys are
                                  sorted by one CTA in shared memory, longer ones by
-                                 a CTA-local radix sort; 256..8192 (32-bit keys),
+                                 one CTA over global memory; 256..8192 (32-bit keys),
                                  256..4096 (64-bit keys); default the maximum */
     void* stream;             /* cudaStream_t */
     void* workspace;          /* optional caller scratch, device, 256-B aligned */
@@ -175,7 +176,7 @@ evosort_status evosort_resolve(size_t n, evosort_dtype dt, int with_values, cons
  * keys: device array of n elements of dtype dt.
  * With p == NULL or p->algo AUTO: arrays of at most small_cap keys take the
  * one-CTA path; otherwise, when a tuned table is loaded, the dispatcher reads
- * a 4096-key strided sample back to the host (synchronising p->stream) and
+ * the class of a 4096-key strided sample, taken on the device, back (synchronising p->stream) and
  * takes the table's entry for the sample's class, and two data-dependent
  * paths come first (keys of at least 2^16 elements): a sample with at most
  * 64 distinct keys is sorted by counting over those values (keys only), and
@@ -185,8 +186,18 @@ evosort_status evosort_resolve(size_t n, evosort_dtype dt, int with_values, cons
  * CUDA graph; calls with explicit parameters (or no table) stay
  * asynchronous.  In every radix sort the passes rank key - min when the
  * keys' span needs fewer 8-bit digits than their raw digits that vary (a
- * decision taken on the device).  Whatever the path, the result is the one
- * sorted array. */
+ * decision taken on the device).
+ * With 8-bit digits and no tile, ranking or pass kernel asked for, arrays
+ * above the one-CTA path and up to 1.3e6 (64-bit pairs) .. 2.5e6 (32-bit
+ * keys) elements are radix sorted by one cooperative launch (the chain of
+ * launches where the device cannot hold its CTAs at once); AUTO sorts of
+ * fewer than 2^16 elements that it takes read no sample unless the table names
+ * the mergesort for the key type.  Larger AUTO sorts of keys alone try two
+ * partition steps and sorts in shared memory first (keys of at least 2^21
+ * elements with a table, which read one more small result back, of 2^23
+ * without, which stay asynchronous), in the same scratch memory, and fall
+ * back to the radix passes where the keys do not spread.  Whatever the path,
+ * the result is the one sorted array. */
 evosort_status evosort_sort(void* keys, size_t n, evosort_dtype dt, const evosort_params* p);
 
 /* Out-of-place variant of evosort_sort (Algorithm 5 with the same paths):
@@ -240,7 +251,8 @@ evosort_status evosort_sort_host_batch(const void* const* keys_in, void* const* 
  * independently, in place, for i in [0, nseg), in one persistent launch
  * (after three small list-building kernels).  Short segments are sorted by
  * one warp in registers, medium ones by one CTA in shared memory, long ones
- * by a CTA-local LSD radix sort (Algorithms 4a/4b) over global memory.
+ * by one CTA that cuts them by their key range and sorts the parts in shared
+ * memory (LSD radix passes, Algorithms 4a/4b, where that separates them not).
  *   keys    DEVICE array of total keys of dtype dt
  *   total   number of keys, which must equal offsets[nseg]
  *   offsets DEVICE array of nseg + 1 uint64: offsets[0] == 0, non-decreasing,
@@ -286,7 +298,7 @@ evosort_status evosort_range_histogram(const void* keys, size_t n, evosort_dtype
 /* ---- Dispatcher and tuned table (Algorithm 5, AdaptivePartitionSort) ----
  * With params == NULL or params->algo == EVOSORT_ALGO_AUTO and a non-empty
  * table, a sort call classifies its input from a strided sample of 4096 keys
- * (one small synchronous device-to-host copy on the call's stream) and uses
+ * (one kernel and a small synchronous copy on the call's stream) and uses
  * the table entry for (dtype, size bucket = floor(log2 n), class): the nearest
  * bucket of the same class, else of the RANDOM class, else the defaults.  The
  * caller's stream and workspace are kept.  With an empty table nothing is

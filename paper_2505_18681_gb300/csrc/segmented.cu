@@ -4,15 +4,14 @@
 //   warp tier   (len < warp cap)     one warp, keys in registers, bitonic
 //                                    network across the warp's lanes (warp cap
 //                                    32..256, a tuning parameter);
-//   block tier  (len <= block cap)   one CTA, keys in shared memory, the
-//                                    insertion-run + merge sort of Algorithm 3;
-//   large tier  (len >  block cap)   one CTA runs the LSD radix sort of
-//                                    Algorithms 4a/4b over the segment in global
-//                                    memory: one read for all digit histograms,
-//                                    then per 8-bit digit a stable tile-by-tile
-//                                    scatter.  A single CTA walks the tiles in
-//                                    order, so running digit offsets replace the
-//                                    device-wide look-back;
+//   block tier  (len <= block cap)   one CTA, keys in shared memory, sorted by
+//                                    bins over their range (bin_sort.cuh; floats
+//                                    by bins over their values);
+//   large tier  (len >  block cap)   one CTA cuts the segment into parts by its
+//                                    sampled range, moves the keys there once
+//                                    and sorts runs of parts in shared memory
+//                                    (cta_sort.cuh; the LSD passes of Algorithms
+//                                    4a/4b where two cuts do not separate them);
 //   giant tier  (len >= giant)       the device-wide radix sort, one segment at
 //                                    a time, before the persistent launch (one
 //                                    CTA per segment would leave the rest of the
@@ -22,6 +21,14 @@
 // segments are the head of that list: the host reads the list's length
 // histogram (one small synchronous copy), sorts the head segments with the
 // device-wide path and has K8 start after them.
+//
+// What bounds K8: in the large tier the shared-memory atomics and accesses per
+// key of three steps (count, move, bin sort) by two CTAs of 512 threads per SM;
+// in the block tier the barriers of one bin sort per segment.  Before, the
+// large tier made a stable pass per digit over global memory and the block
+// tier merged: 10,000 int32 segments up to 1e6 keys (9.1e8 keys) 17.2 -> 9.2
+// ms, 20,000 int64 ones up to 8,000 (2.6e7 keys) 1.80 -> 0.56 ms, 3,000
+// float64 ones up to 1e5 (3.5e7 keys) 1.64 -> 0.79 ms.
 #include <algorithm>
 #include <vector>
 
