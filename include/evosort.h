@@ -135,7 +135,10 @@ typedef struct {
                                  by one CTA in shared memory in a single launch
                                  with no scratch memory (the GPU form of the
                                  paper's small-array fallback, Algorithm 5);
-                                 0 = default: 4096 when algo is AUTO, else off;
+                                 0 = default: 4096 when algo is AUTO, else off
+                                 (a call that also names no scratch and no
+                                 parameter of the radix kernels: 8192, and 15360
+                                 32-bit keys without values);
                                  1 = off; 2..8192 = that cut-over, whatever the
                                  algo */
     long long seg_giant;      /* segmented sort: segments longer than this many

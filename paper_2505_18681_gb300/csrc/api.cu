@@ -670,6 +670,16 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
         return cudaStreamIsCapturing(p ? (cudaStream_t)p->stream : nullptr, &cap) == cudaSuccess &&
                cap == cudaStreamCaptureStatusNone;
     };
+    if (automatic && fused && !(p && (p->small_cap || p->digit_bits || p->workspace)) && n <= small_auto_keys(w, pairs) &&
+        (!table_nonempty() || needs_no_sample())) {
+        // one CTA's bins are still done before the one-launch radix sort's
+        // barriers over the grid
+        Plan sp;
+        int rc0 = resolve(p, dt, pairs, &sp, &err, n);
+        if (rc0 == EVOSORT_OK)
+            rc0 = small_sort(in, out, vin, vout, n, dt, sp, p ? (cudaStream_t)p->stream : nullptr, &err);
+        return finish(rc0, err);
+    }
     if (automatic && table_nonempty() && !needs_no_sample()) {
         void* st = p ? p->stream : nullptr;
         const bool desc = p && p->descending;

@@ -42,6 +42,9 @@ enum : int { HYBRID_OFF = 0, HYBRID_ASYNC = 1, HYBRID_SYNC = 2 };
 // default and largest cut-over, in keys.
 constexpr int kSmallDefault = 4096;
 constexpr int kSmallMax = 8192;
+// Largest array that the dispatcher gives to one CTA by itself, where the caller
+// names neither a cut-over, scratch nor a parameter of the radix kernels.
+size_t small_auto_keys(int w, bool pairs);
 int small_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n, int dt, const Plan& pl,
                cudaStream_t s, std::string* err);
 

@@ -31,7 +31,7 @@
 
 namespace evosort {
 
-constexpr int kBinMax = 1 << 15;     // most bins
+constexpr int kBinMax = 1 << 16;     // most bins
 constexpr int kBinThreadKeys = 31;   // longest bin one thread sorts (2^k - 1)
 constexpr int kBinWarpKeys = 16;     // keys per lane of the warp sort
 
@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t cut_range(unsigned long long width, uint32_t
     }
     const int z = __clzll((long long)width);
     *lz = z;
-    if (width < (unsigned long long)parts) {   // (parts <= kBinMax, so z >= 49)
+    if (width < (unsigned long long)parts) {   // (parts <= kBinMax, so z >= 48)
         *mult = 1u << (64 - z);
         return (uint32_t)width + 1u;
     }
@@ -472,14 +472,21 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
 
     // ---- exclusive scan of the bins.  A count that ran over its 8 bits shows
     // in the total: it takes 256 from its own and gives at most one away.
-    uint32_t sum = 0, any = 0, multi = 0;   // multi: words with a bin of two or more keys
+    uint32_t sum = 0, any = 0, widest = 0, multi = 0;   // multi: words with a bin of two or more keys
 #pragma unroll
     for (int j = 0; j < WPT / 4; ++j) {
         const uint4 q = mine[j];
-        sum = __dp4a(q.x, 0x01010101u, sum);
-        sum = __dp4a(q.y, 0x01010101u, sum);
-        sum = __dp4a(q.z, 0x01010101u, sum);
-        sum = __dp4a(q.w, 0x01010101u, sum);
+        if constexpr (OWN) {
+            const uint32_t x = __dp4a(q.x, 0x01010101u, 0u), y = __dp4a(q.y, 0x01010101u, 0u);
+            const uint32_t z = __dp4a(q.z, 0x01010101u, 0u), t = __dp4a(q.w, 0x01010101u, 0u);
+            sum += (x + y) + (z + t);
+            widest = max(max(widest, max(x, y)), max(z, t));
+        } else {
+            sum = __dp4a(q.x, 0x01010101u, sum);
+            sum = __dp4a(q.y, 0x01010101u, sum);
+            sum = __dp4a(q.z, 0x01010101u, sum);
+            sum = __dp4a(q.w, 0x01010101u, sum);
+        }
         any |= q.x | q.y | q.z | q.w;
         if (q.x & 0xFEFEFEFEu) multi |= 1u << (4 * j);
         if (q.y & 0xFEFEFEFEu) multi |= 2u << (4 * j);
@@ -493,12 +500,17 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
         if (lane >= o) inc += y;
     }
     if (lane == 31) sh.wsum[warp] = inc;
-    // a word's counts must stay below 64 in all: bins below 16
+    // a word's counts must stay below 64 in all: bins below 16, or, where the
+    // other way is the slower one, every word counted
     // With positions equal keys have to be put in order too, and a narrow range
     // takes the caller two radix passes at most: bins below 8 there (4,000
-    // floats with 8 to 15 equal ones among them: 14.3 us so, 22.5 by passes).
-    const uint32_t limit = IDX && width < 65536ull ? 0xF8F8F8F8u : 0xF0F0F0F0u;
-    const bool heavy = __syncthreads_or((any & limit) != 0u);
+    // floats with 8 to 15 equal ones among them: 14.3 us by insertion, 22.5 by passes).
+    // Positions arrive in no order, which insertion pays for with the square of
+    // the bin: bins below 16 where the other way is short too (16 values among
+    // 300 pairs: 5.0 us by passes, 16.7 by insertion; 8,192 pairs of floats with
+    // 20 equal ones at most: 36 and 16.5).
+    const bool few = IDX && width < 65536ull, strict = !OWN || few || (IDX && n <= 4096);
+    const bool heavy = __syncthreads_or(strict ? (any & (few ? 0xF8F8F8F8u : 0xF0F0F0F0u)) != 0u : widest > 63u);
     uint32_t run = inc - sum;
     {
         const uint32_t v = lane < NW ? sh.wsum[lane] : 0u;

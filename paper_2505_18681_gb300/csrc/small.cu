@@ -32,15 +32,18 @@ namespace {
 
 constexpr int kSmallThreads = 512;
 static_assert(kSmallMax <= 16 * kSmallThreads, "largest compiled shape");
+// A second size of CTA for 32-bit keys alone (64-bit keys and values leave no
+// room in 64 registers, or in shared memory).
+constexpr int kSmallWideThreads = 1024;
+constexpr int kSmallWideKpt = 15;   // (a place in the bins has 14 bits)
 __host__ __device__ constexpr size_t small_up(size_t x) { return (x + 15) / 16 * 16; }
 constexpr int kSmallRun = 16;   // longest insertion-sorted base run
 
 // KPT keys per thread at most, WPT words of four bins per thread.
-template <typename U, bool PAIRS, bool FLT, int KPT, int WPT>
-__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, U* out, const uint32_t* vin,
+template <typename U, bool PAIRS, bool FLT, int NT, int KPT, int WPT>
+__global__ void __launch_bounds__(NT) small_sort_kernel(const U* in, U* out, const uint32_t* vin,
                                                                     uint32_t* vout, int n, KeyMap map, int tins) {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int NT = kSmallThreads;
     __shared__ BinShared<U, NT> sh;
     // keys, the bins' words or the merge sort's second array, values and
     // input positions or the merge sort's second values
@@ -117,9 +120,28 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
         int which = 0;
         if (lead) {
             smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, bits - 16, 2, counts, sh.wsum);   // back in k0
-            bool down = false;
-            for (int i = tid + 1; i < n; i += NT) down |= k0[i] < k0[i - 1];
-            sorted = !__syncthreads_or(down);
+            // the few keys that share them and differ: exchanges of neighbours,
+            // which keep equal keys in order (90% zeros among 10,000 int32 keys)
+            bool quiet = false;
+            for (int r = 0; r < 12 && !sorted; ++r) {
+                bool moved = false;
+                for (int i = 2 * tid + (r & 1); i + 1 < n; i += 2 * NT) {
+                    const U a = k0[i], b = k0[i + 1];
+                    if (b < a) {
+                        k0[i] = b;
+                        k0[i + 1] = a;
+                        if (PAIRS) {
+                            const uint32_t va = v0[i];
+                            v0[i] = v0[i + 1];
+                            v0[i + 1] = va;
+                        }
+                        moved = true;
+                    }
+                }
+                const bool still = !__syncthreads_or(moved);
+                sorted = still && quiet;   // neither the even nor the odd pairs moved
+                quiet = still;
+            }
         }
         if (!sorted) {   // (equal keys are still in input order)
             int rounds = 1;
@@ -139,25 +161,26 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const U* in, 
     }
 }
 
-// Most keys of each compiled shape (keys per thread, words per thread).
+// Most keys of each compiled shape (keys per thread, words per thread); 32-bit
+// keys alone have one more, of 1,024 threads.
 #define EVOSORT_SMALL_SHAPES(X) X(2, 4) X(8, 12) X(16, 12)
 
-template <typename U, bool PAIRS, bool FLT, int KPT, int WPT>
+template <typename U, bool PAIRS, bool FLT, int NT, int KPT, int WPT>
 cudaError_t launch_small_shape(const void* in, void* out, const uint32_t* vin, uint32_t* vout, int n, KeyMap map,
                                int tins, cudaStream_t s) {
-    auto kern = small_sort_kernel<U, PAIRS, FLT, KPT, WPT>;
+    auto kern = small_sort_kernel<U, PAIRS, FLT, NT, KPT, WPT>;
     auto bytes = [](int m) {
-        return small_up(m * sizeof(U)) + small_up(bin_scratch_bytes(m, (int)sizeof(U), WPT * kSmallThreads)) +
-               (PAIRS ? (size_t)m * 8 : 0) + (size_t)kSmallThreads / 32 * 512;
+        return small_up(m * sizeof(U)) + small_up(bin_scratch_bytes(m, (int)sizeof(U), WPT * NT)) +
+               (PAIRS ? (size_t)m * 8 : 0) + (size_t)NT / 32 * 512;
     };
     static bool configured = false;
     if (!configured) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)bytes(KPT * kSmallThreads));
+                                                   (int)bytes(KPT * NT));
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    kern<<<1, kSmallThreads, bytes(n), s>>>((const U*)in, (U*)out, vin, vout, n, map, tins);
+    kern<<<1, NT, bytes(n), s>>>((const U*)in, (U*)out, vin, vout, n, map, tins);
     return cudaGetLastError();
 }
 
@@ -165,19 +188,32 @@ template <typename U, bool PAIRS, bool FLT>
 cudaError_t launch_small(const void* in, void* out, const uint32_t* vin, uint32_t* vout, int n, KeyMap map,
                          int tins, cudaStream_t s) {
 #define EVOSORT_CASE(K, W) \
-    if (n <= K * kSmallThreads) return launch_small_shape<U, PAIRS, FLT, K, W>(in, out, vin, vout, n, map, tins, s);
+    if (n <= K * kSmallThreads) return launch_small_shape<U, PAIRS, FLT, kSmallThreads, K, W>(in, out, vin, vout, n, map, tins, s);
     EVOSORT_SMALL_SHAPES(EVOSORT_CASE)
 #undef EVOSORT_CASE
+    if constexpr (sizeof(U) == 4 && !PAIRS)
+        if (n <= kSmallWideKpt * kSmallWideThreads)
+            return launch_small_shape<U, PAIRS, FLT, kSmallWideThreads, kSmallWideKpt, 12>(in, out, vin, vout, n, map,
+                                                                                           tins, s);
     return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
+// Against the one-launch radix sort, whose barriers over the grid take it 37 us
+// for 32-bit and 57 to 64 us for 64-bit keys at these sizes: 10,000 uniform
+// int32 keys 9.5 us, 15,360 12.0, 8,192 uniform int64 keys 11.4, with values
+// 15.5.  Keys that the bins do not separate are about even (Zipf, 8,192 int32 keys
+// 26.6 and 26.8 us, 15,360 42 and 31).
+size_t small_auto_keys(int w, bool pairs) {
+    return w == 4 && !pairs ? (size_t)kSmallWideKpt * kSmallWideThreads : (size_t)kSmallMax;
+}
+
 int small_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n, int dt, const Plan& pl,
                cudaStream_t s, std::string* err) {
     const int w = dtype_bytes(dt);
     const bool pairs = vout != nullptr;
-    if (n > (size_t)kSmallMax) {
+    if (n > small_auto_keys(w, pairs)) {
         *err = "small-array path: more keys than it holds";
         return EVOSORT_ERR_INVALID;
     }

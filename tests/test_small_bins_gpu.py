@@ -97,3 +97,29 @@ def test_integers(evo, dtype, kind):
 def test_floats(evo, dtype, kind):
     for n in SIZES:
         check(evo, floats(kind, n, dtype))
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.float32, np.int64], ids=["int32", "float32", "int64"])
+@pytest.mark.parametrize("kind", ["spread", "few", "clump", "late", "ends", "normal", "specials"])
+def test_arrays_the_dispatcher_gives_to_one_cta(evo, dtype, kind):
+    """Above the default cut-over, with the choice left to the library: the
+    last size of each width that one CTA takes and the first that it does not."""
+    if (dtype == np.float32) != (kind in ("normal", "specials")):
+        pytest.skip("a kind of the other key types")
+    for n in (4097, 8191, 8192, 8193, 12289, 15359, 15360, 15361):
+        a = floats(kind, n, dtype) if dtype == np.float32 else ints(kind, n, dtype)
+        x = torch.from_numpy(a.copy()).cuda()
+        y, d = torch.empty_like(x), torch.empty_like(x)
+        evo.sync()
+        evo.profile(True)
+        try:
+            evo.sort(x, out=y)
+            evo.sync()
+            kinds = [r["kind"] for r in evo.profile_read()]
+        finally:
+            evo.profile(False)
+        evo.sort(x, out=d, descending=True)
+        evo.sync()
+        want = oracle.radix_sort(a)
+        assert np.array_equal(bits(y), bits(want)) and np.array_equal(bits(d), bits(want)[::-1]), n
+        assert (kinds == ["small"]) == (n <= (15360 if a.itemsize == 4 else 8192)), n
