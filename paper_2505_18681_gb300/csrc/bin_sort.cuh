@@ -18,8 +18,8 @@
 // fewer keys to sort inside bins.  1e9 int32 / int64 keys, all groups: 5.3 /
 // 7.3 ms with 10,240 32-bit counters.
 //
-// Where the stretches do not separate the keys (a word of 32 keys or more),
-// block_bin_sort_wide takes over: 32-bit counters, bins of up to 32 *
+// Where the stretches do not separate the keys (a bin of 16 keys or more),
+// the caller's own way (OWN) or block_bin_sort_wide takes over: 32-bit counters, bins of up to 32 *
 // kBinWarpKeys keys sorted by one warp each (bitonic), and if some bin is larger
 // still the merge sort of Algorithm 3, so any input is sorted in bounded time.
 #pragma once

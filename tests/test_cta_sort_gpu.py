@@ -84,7 +84,7 @@ def test_float_segments_cut_by_value(evo, dtype, kind):
     if kind == "orders":
         x = np.ldexp(x, r.integers(-100, 100, n))
     elif kind == "specials":
-        x = np.choose(r.integers(0, 12, n), [x * np.finfo(dtype).max / 16, np.inf, -np.inf, np.nan, -np.nan, 0.0, -0.0] + [x] * 5)
+        x = np.choose(r.integers(0, 12, n), [x * (np.finfo(dtype).max / 64), np.inf, -np.inf, np.nan, -np.nan, 0.0, -0.0] + [x] * 5)
     elif kind == "infinite":
         x = np.where(r.random(n) < 0.5, np.inf, -np.inf)
     x = x.astype(dtype)
