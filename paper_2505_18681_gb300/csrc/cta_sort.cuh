@@ -10,12 +10,14 @@
 //                    still too large is cut once more, over its own range;
 //   cta_radix_sort   the LSD radix passes of Algorithms 4a/4b by one CTA, for
 //                    what two cuts do not separate (many equal keys among
-//                    others).  The CTA walks the tiles in order, so running
-//                    digit offsets replace a look-back.
+//                    others) and for runs longer than 32-bit counters hold.
+//                    The CTA walks the tiles in order, so running digit
+//                    offsets replace a look-back.
 #pragma once
 
 #include "bin_sort.cuh"
 #include "common.cuh"
+#include "seg_tiers.h"
 
 namespace evosort {
 
@@ -97,17 +99,22 @@ __device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int
 
 // LSD radix sort of the len mapped keys in a (other buffer b); the sorted
 // keys, through out(), end in fin (a or b).  8-bit digits; digits that are
-// equal in all keys are skipped.
-template <typename U, typename M>
-__device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, uint32_t len, M out, unsigned char* smem,
-                                            CtaShared<U>& sh) {
+// equal in all keys are skipped.  I counts keys: 32 bits for runs of at most
+// kSegCutKeys, 64 bits for any.
+template <typename I, typename U, typename M>
+__device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, unsigned char* smem, CtaShared<U>& sh) {
     constexpr int NP = sizeof(U);
     constexpr int BINS = 256;
     constexpr int KPT = 8;
     constexpr uint32_t TILE = kCtaThreads * KPT;
-    uint32_t* s_hist = (uint32_t*)smem;                 // NP * BINS
-    uint32_t* s_run = s_hist + NP * BINS;               // BINS running offsets
-    uint32_t* s_excl = s_run + BINS;                    // BINS tile offsets
+    static_assert(sizeof(I) == 8 || kSegCutKeys + 4u * kCtaThreads <= 0xFFFFFFFFull, "an unrolled step past the end");
+    static_assert(sizeof(I) == 8 || kSegCutKeys + TILE <= 0xFFFFFFFFull, "a tile past the end");
+    static_assert((NP + 1) * BINS * sizeof(I) + BINS * 8 + kCtaWarps * BINS * 6 + TILE * sizeof(U) <= cta_buf_bytes<U>(),
+                  "shared memory");
+    static_assert(NP <= kCtaWarps, "the long runs' counts in the match masks' room");
+    I* s_hist = (I*)smem;                               // NP * BINS
+    I* s_run = s_hist + NP * BINS;                      // BINS running offsets
+    uint32_t* s_excl = (uint32_t*)(s_run + BINS);       // BINS tile offsets
     uint32_t* s_tcnt = s_excl + BINS;                   // BINS tile counts
     uint32_t* s_match = s_tcnt + BINS;                  // warps * BINS match masks
     uint16_t* s_whist = (uint16_t*)(s_match + kCtaWarps * BINS);   // warps * BINS
@@ -116,13 +123,32 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, uint32_t len, M 
     for (int i = tid; i < NP * BINS; i += kCtaThreads) s_hist[i] = 0;
     if (tid < NP) sh.active[tid] = 0;
     __syncthreads();
+    auto count = [&](const U* keys, uint32_t m, uint32_t* hist) {
 #pragma unroll 4
-    for (uint32_t i = tid; i < len; i += kCtaThreads) {
-        const U k = a[i];
+        for (uint32_t i = tid; i < m; i += kCtaThreads) {
+            const U k = keys[i];
 #pragma unroll
-        for (int p = 0; p < NP; ++p) atomicAdd(&s_hist[p * BINS + digit_of(k, 8 * p, 0xFFu)], 1u);
+            for (int p = 0; p < NP; ++p) atomicAdd(&hist[p * BINS + digit_of(k, 8 * p, 0xFFu)], 1u);
+        }
+        __syncthreads();
+    };
+    if constexpr (sizeof(I) == 4) {
+        count(a, len, s_hist);
+    } else {
+        // 32-bit counts of a stretch at a time, in the room of the match masks
+        // (64-bit shared atomics queue up on a digit that is equal in all
+        // keys: 2^31 keys of 600 values took 84 s)
+        for (int i = tid; i < NP * BINS; i += kCtaThreads) s_match[i] = 0u;
+        __syncthreads();
+        for (I at = 0; at < len; at += kSegCutKeys) {
+            count(a + at, (uint32_t)(len - at < kSegCutKeys ? len - at : kSegCutKeys), s_match);
+            for (int i = tid; i < NP * BINS; i += kCtaThreads) {
+                s_hist[i] += s_match[i];
+                s_match[i] = 0u;
+            }
+            __syncthreads();
+        }
     }
-    __syncthreads();
     for (int i = tid; i < NP * BINS; i += kCtaThreads)
         if (s_hist[i] != 0 && s_hist[i] != len) sh.active[i / BINS] = 1;
     __syncthreads();
@@ -135,13 +161,18 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, uint32_t len, M 
         if (!sh.active[p]) continue;
         const int shift = 8 * p;
         {
-            const uint32_t c = tid < BINS ? s_hist[p * BINS + tid] : 0u;
-            uint32_t tot;
-            const uint32_t ex = block_exclusive_scan<kCtaThreads>(c, sh.scan, &tot);
+            const I c = tid < BINS ? s_hist[p * BINS + tid] : (I)0;
+            I tot;
+            I* scan;
+            if constexpr (sizeof(I) == 4)
+                scan = sh.scan;
+            else
+                scan = (I*)s_match;   // (cleared again by the first tile)
+            const I ex = block_exclusive_scan<kCtaThreads, I>(c, scan, &tot);
             if (tid < BINS) s_run[tid] = ex;
         }
         __syncthreads();
-        for (uint32_t t0 = 0; t0 < len; t0 += TILE) {
+        for (I t0 = 0; t0 < len; t0 += TILE) {
             const int valid = len - t0 < TILE ? (int)(len - t0) : (int)TILE;
             uint16_t* wh = s_whist + warp * BINS;
             uint32_t* wm = s_match + warp * BINS;
@@ -213,13 +244,14 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, uint32_t len, M 
         src = dst;
         dst = t;
     }
-    for (uint32_t i = tid; i < len; i += kCtaThreads) fin[i] = out(src[i]);
+    for (I i = tid; i < len; i += kCtaThreads) fin[i] = out(src[i]);
     __syncthreads();
 }
 
 // Sort of the len keys of src: in() maps a key on its load, out() on its last
 // store.  The parts are laid out in part (as long as src); the sorted keys end
-// in fin, which is src or part.  LEVEL 0 cuts too large parts again.
+// in fin, which is src or part.  LEVEL 0 cuts too large parts again.  len is at
+// most kSegCutKeys: the counters are of 32 bits.
 template <typename U, int LEVEL, typename MI, typename MO>
 __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
                                                unsigned char* smem, CtaShared<U>& sh);
@@ -240,6 +272,8 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
     constexpr int KPT = cta_kpt<U>();
     constexpr int CAP = cta_cap<U>();
     constexpr uint32_t TILE = CAP;
+    static_assert(kSegCutKeys + TILE <= 0xFFFFFFFFull && kSegCutKeys + 16u * kCtaThreads <= 0xFFFFFFFFull,
+                  "a step past the end");
     U* s_key = (U*)smem;                                                  // tile buffer, or a local sort's first
     uint32_t* s_cnt = (uint32_t*)(smem + (size_t)CAP * sizeof(U));        // tile counts (the second buffer)
     uint32_t* s_at = s_cnt + kCtaParts;
@@ -344,7 +378,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
     if (!one_value && sh.longest > (uint32_t)CAP && sh.longest > len / 2u) {
         for (uint32_t i = tid; i < len; i += kCtaThreads) src[i] = in(src[i]);
         __syncthreads();
-        cta_radix_sort<U>(src, part, fin, len, out, smem, sh);
+        cta_radix_sort<uint32_t, U>(src, part, fin, len, out, smem, sh);
         return;
     }
 
@@ -439,7 +473,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
                 cta_split_again<U>(part + s, other, fin + s, n, out, smem, sh);
             } else {
                 __syncthreads();
-                cta_radix_sort<U>(part + s, other, fin + s, n, out, smem, sh);
+                cta_radix_sort<uint32_t, U>(part + s, other, fin + s, n, out, smem, sh);
             }
         } else if (n > 0) {
             U key[KPT];

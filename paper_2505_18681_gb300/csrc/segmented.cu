@@ -12,6 +12,9 @@
 //                                    and sorts runs of parts in shared memory
 //                                    (cta_sort.cuh; the LSD passes of Algorithms
 //                                    4a/4b where two cuts do not separate them);
+//   long tier   (len >= 2^31)        the LSD passes with 64-bit counters by one
+//                                    CTA (seg_tiers.h), for segments that the
+//                                    giant tier did not take;
 //   giant tier  (len >= giant)       the device-wide radix sort, one segment at
 //                                    a time, before the persistent launch (one
 //                                    CTA per segment would leave the rest of the
@@ -36,6 +39,7 @@
 #include "api_internal.h"
 #include "common.cuh"
 #include "cta_sort.cuh"
+#include "seg_tiers.h"
 #include "smem_sort.cuh"
 
 namespace evosort {
@@ -54,7 +58,8 @@ struct SegArgs {
     KeyMap map;
     void* tmp;          // scratch of total keys (large-tier ping-pong)
     uint32_t* hdr;      // [0..kNB) bucket counts, [kNB..2kNB) bucket cursors,
-                        // [2kNB] single items, [2kNB+1] warp-tier segments, [2kNB+2] work counter
+                        // [2kNB] single items, [2kNB+1] warp-tier segments, [2kNB+2] work counter,
+                        // [2kNB+3] long-tier segments
     uint32_t* order;    // nseg entries: segment ids, longest first
     uint32_t* status;
     int block_cap;      // keys one CTA sorts in shared memory
@@ -89,7 +94,7 @@ __global__ void seg_count(SegArgs a) {
 // K7b: bucket cursors in descending length order, item counts.
 __global__ void seg_scan(SegArgs a) {
     if (threadIdx.x != 0) return;
-    uint32_t pos = 0, single = 0, warp = 0;
+    uint32_t pos = 0, single = 0, warp = 0, longs = 0;
     for (int b = kNB - 1; b >= 1; --b) {
         a.hdr[kNB + b] = pos;
         pos += a.hdr[b];
@@ -97,10 +102,12 @@ __global__ void seg_scan(SegArgs a) {
             single += a.hdr[b];
         else
             warp += a.hdr[b];
+        if (b >= kSegLongLog2) longs += a.hdr[b];
     }
     a.hdr[2 * kNB] = single;
     a.hdr[2 * kNB + 1] = warp;
     a.hdr[2 * kNB + 2] = 0;
+    a.hdr[2 * kNB + 3] = longs;
 }
 
 // K7c: scatter segment ids into the work list.
@@ -157,13 +164,15 @@ __global__ void __launch_bounds__(kSB, 2) seg_sort(SegArgs a) {
     const uint32_t single = a.hdr[2 * kNB];
     const uint32_t nwarp = a.hdr[2 * kNB + 1];
     const uint32_t nbatch = (nwarp + kSW - 1) / kSW;
+    // the head of the list: sorted by the device-wide path, or left to seg_long
+    const uint32_t skip = max(a.skip, a.hdr[2 * kNB + 3]);
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(&a.hdr[2 * kNB + 2], 1u);
         __syncthreads();
         const uint32_t item = s_item;
         __syncthreads();
         if (item >= single + nbatch) break;
-        if (item < a.skip) continue;   // sorted by the device-wide path
+        if (item < skip) continue;
         if (item < single) {
             const uint32_t seg = a.order[item];
             const uint64_t lo = a.off[seg], len = a.off[seg + 1] - lo;
@@ -181,6 +190,25 @@ __global__ void __launch_bounds__(kSB, 2) seg_sort(SegArgs a) {
                 warp_tier<U>(a, lo, (int)(a.off[seg + 1] - lo), in, out);
             }
         }
+    }
+}
+
+// Long tier: the head of the work list after the giant segments, one CTA per
+// segment.  Launched only for batches that can hold such a segment; a kernel
+// of its own, so that the other tiers keep their registers.
+template <typename U>
+__global__ void __launch_bounds__(kSB) seg_long(SegArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ CtaShared<U> sh;
+    const uint32_t longs = a.hdr[2 * kNB + 3];
+    for (uint32_t item = a.skip + blockIdx.x; item < longs; item += gridDim.x) {
+        const uint32_t seg = a.order[item];
+        const uint64_t lo = a.off[seg];
+        const unsigned long long len = a.off[seg + 1] - lo;
+        U* keys = (U*)a.keys + lo;
+        for (unsigned long long i = threadIdx.x; i < len; i += kSB) keys[i] = map_fwd(keys[i], a.map);
+        __syncthreads();
+        cta_radix_sort<unsigned long long, U>(keys, (U*)a.tmp + lo, keys, len, GeneralOut<U>(a.map), smem, sh);
     }
 }
 
@@ -275,6 +303,16 @@ int segmented_sort(void* keys, size_t total, const uint64_t* off, size_t nseg, i
             if (e == cudaSuccess) {
                 kern<<<(unsigned)(sms * resident[wi][fi]), kSB, smem, s>>>(a);
                 e = cudaGetLastError();
+            }
+            if (e == cudaSuccess && total > kSegCutKeys) {
+                void (*const longk)(SegArgs) = w == 4 ? seg_long<uint32_t> : seg_long<uint64_t>;
+                e = cudaFuncSetAttribute(longk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                const size_t most = total >> kSegLongLog2;   // such segments
+                if (e == cudaSuccess) {
+                    longk<<<(unsigned)(most < (size_t)sms ? most : (size_t)sms), kSB, smem, s>>>(a);
+                    e = cudaGetLastError();
+                    count_launches(1);
+                }
             }
         }
     }
