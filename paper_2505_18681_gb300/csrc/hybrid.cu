@@ -880,7 +880,13 @@ __global__ void __launch_bounds__(kHybThreads, 3) hybrid_count_b(HybArgs a) {
 template <typename U>
 __global__ void __launch_bounds__(kHybThreads) hybrid_scan_b(HybArgs a) {
     chain_wait();
-    if (!hyb_on(a.ctl)) return;
+    // Other CTAs of this launch may give the path up while this one starts: one
+    // thread reads the verdict so far for all of them, or some would leave and
+    // the rest wait at the barriers below.
+    __shared__ bool s_on;
+    if (threadIdx.x == 0) s_on = hyb_on(a.ctl);
+    __syncthreads();
+    if (!s_on) return;
     __shared__ uint32_t s_scr[kHybThreads / 32 + 1];
     const int bin = blockIdx.x, tid = threadIdx.x;
     constexpr int PER = kHybBins / kHybThreads;

@@ -62,6 +62,8 @@ def gen(name, n, dtype, seed=3):
         x[n // 2 + 1] = (1 << 62) + 7
     elif name == "crowded":     # one key in fifty in a stretch of 2^20 values of the whole range
         x = torch.where(x % 50 == 0, (x >> 44) + (1 << 40), x)
+    elif name == "pressed":     # the same with one key in 120: the sample accepts it, a bucket is too long
+        x = torch.where(x % 120 == 0, (x >> 44) + (1 << 40), x)
     elif name == "frequent":    # one value held by 15 % of the keys, the others spread over 2^20 values
         x = torch.where((x >> 8) % 100 < 15, torch.full_like(x, 77), (x >> 44) & 0xFFFFF)
     elif name == "powers":      # magnitudes spread over every binary order
@@ -156,3 +158,25 @@ def test_captured_graph_decides_anew_for_new_keys(evo):
         g.replay()
         torch.cuda.synchronize()
         assert np.array_equal(bits(y), bits(oracle.radix_sort(host(x)))), name
+
+
+@pytest.mark.parametrize("table", [False, True], ids=["async", "table"])
+@pytest.mark.parametrize("dtype", [torch.int64, torch.uint64], ids=str)
+def test_given_up_after_the_counts(evo, dtype, table):
+    """The sample accepts the keys and the counts refuse them: the radix passes
+    sort them, in the scratch that the partition sort cleared, and sort other
+    keys right after."""
+    x = gen("pressed", N, torch.int64).view(dtype)
+    want = bits(oracle.radix_sort(host(x)))
+    if table:
+        for t in TABLES:
+            evo.table_load(t)
+    y, z = torch.empty_like(x), x.clone()
+    for _ in range(3):
+        assert taken(evo, lambda: evo.sort(x, out=y)) == (False, True)
+        assert np.array_equal(bits(y), want)
+        y.zero_()
+    evo.sort(z)
+    evo.sort(x, out=y, descending=True)
+    evo.sync()
+    assert np.array_equal(bits(z), want) and np.array_equal(bits(y), want[::-1])
