@@ -454,10 +454,10 @@ evosort_status evosort_sync(void* stream);
  * the paper (host memory needs no such call there). */
 evosort_status evosort_release(void);
 
-/* Poll limit of the bounded device-side waits on look-back slots, for tests
- * of the failure path and for debugging (the paper has no counterpart).
- * polls == 0 restores the built-in limit (2^22 polls, about a second).  A
- * wait that runs out records EVOSORT_ERR_TIMEOUT for the next evosort_sync
+/* Poll limit of the bounded device-side waits on look-back slots and at the
+ * one-launch radix sort's barriers over the grid, for tests of the failure
+ * path and for debugging (the paper has no counterpart).  polls == 0 restores
+ * the built-in limit (2^22 polls, about a second).  A wait that runs out records EVOSORT_ERR_TIMEOUT for the next evosort_sync
  * and its kernel returns; that sort's output is then invalid.  Applies to
  * sorts enqueued after the call, process-wide. */
 void evosort_set_wait_limit(uint32_t polls);

@@ -349,8 +349,8 @@ def release() -> None:
 
 
 def set_wait_limit(polls: int) -> None:
-    """Poll limit of the device-side look-back waits (0 = built-in default);
-    for tests of the failure path."""
+    """Poll limit of the device-side waits (look-back, barriers of the
+    one-launch radix sort; 0 = built-in default); for tests of the failure path."""
     library().evosort_set_wait_limit(int(polls))
 
 

@@ -48,8 +48,8 @@ size_t small_auto_keys(int w, bool pairs);
 int small_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n, int dt, const Plan& pl,
                cudaStream_t s, std::string* err);
 
-// Poll limit of the bounded device-side waits (look-back slots); set by
-// evosort_set_wait_limit, 0 = the built-in default.
+// Poll limit of the bounded device-side waits (look-back slots, the one-launch
+// radix sort's barriers); set by evosort_set_wait_limit, 0 = the built-in default.
 uint32_t wait_limit();
 
 void set_error(const std::string& msg);

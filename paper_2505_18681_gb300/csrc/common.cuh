@@ -16,8 +16,8 @@ enum : uint32_t { ST_TIMEOUT = 1u, ST_BAD_OFFSETS = 2u, ST_RANGE = 4u };
 
 // Bounded waits: polls before a kernel gives up, records ST_TIMEOUT and
 // proceeds (its output is then invalid but the context lives).  Look-back
-// waits take their limit from the launch (evosort_set_wait_limit, default
-// this value); mbarrier waits for the kernel's own bulk copies always use it.
+// waits and the one-launch radix sort's barriers take their limit from the
+// launch (evosort_set_wait_limit, default this value); mbarrier waits for the kernel's own bulk copies always use it.
 constexpr uint32_t kSpinLimit = 1u << 22;
 
 inline int dtype_bytes(int dt) { return (dt == DT_I32 || dt == DT_U32 || dt == DT_F32) ? 4 : 8; }

@@ -56,6 +56,7 @@ struct FusedArgs {
     uint32_t* bins;             // kFusCount value counts (keys only)
     PassDesc* desc;             // sizeof(U) + 1 entries, for the profile's records
     uint32_t* status;
+    uint32_t limit;             // polls of one barrier
 };
 
 template <typename U, bool PAIRS>
@@ -67,7 +68,9 @@ constexpr size_t fus_smem() {
 }
 
 // Barrier over the grid; step counts them from 1.  False if it ran out of
-// polls; every CTA then gives up, here or at its next barrier.
+// polls (a.limit, as the look-back's waits); every CTA then gives up, here or at
+// its next barrier, which the ones that left never reach.  What a barrier
+// protects is read only after it was complete, so nothing is read too early.
 __device__ __forceinline__ bool fus_barrier(const FusedArgs& a, uint32_t step, int* s_stop) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -78,7 +81,7 @@ __device__ __forceinline__ bool fus_barrier(const FusedArgs& a, uint32_t step, i
         uint32_t polls = 0;
         int stop = 0;
         while (ld_relaxed(word) < want) {
-            if (++polls > kSpinLimit) {
+            if (++polls > a.limit) {
                 atomicOr(a.status, ST_TIMEOUT);
                 stop = 1;
                 break;
@@ -441,6 +444,7 @@ cudaError_t launch_radix_fused(int w, const void* in, void* out, const uint32_t*
     a.bins = (uint32_t*)bins;
     a.desc = desc;
     a.status = status;
+    a.limit = wait_limit();
     const int sms = sm_count();
     if (w == 4) return vout ? launch_fused<uint32_t, true>(a, sms, s) : launch_fused<uint32_t, false>(a, sms, s);
     return vout ? launch_fused<uint64_t, true>(a, sms, s) : launch_fused<uint64_t, false>(a, sms, s);

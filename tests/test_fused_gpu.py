@@ -155,3 +155,27 @@ def test_two_streams_at_once(evo):
         evo.sync(s)
     for x, y in zip(xs, ys):
         assert np.array_equal(bits(y), bits(oracle.radix_sort(host(x))))
+
+
+@pytest.mark.parametrize("pairs", [False, True], ids=["keys", "pairs"])
+@pytest.mark.parametrize("dtype,n", [(torch.int32, 1_000_003), (torch.int64, 20_000), (torch.float64, 700_001)], ids=str)
+def test_barrier_wait_times_out_and_recovers(evo, dtype, n, pairs):
+    """With the poll limit cut to one, the first barrier over the grid runs out:
+    the kernel returns, evosort_sync reports ERR_TIMEOUT, and the next sorts with
+    the default limit match the oracle."""
+    x = gen("uniform", n, dtype)
+    v = torch.arange(n, dtype=torch.int32, device="cuda").view(torch.uint32)
+    y, w = torch.empty_like(x), torch.empty_like(v)
+    sort = (lambda: evo.sort_pairs(x, v, y, w, algo="radix")) if pairs else (lambda: evo.sort(x, out=y, algo="radix"))
+    count, kinds = launches(evo, sort)
+    assert count == 1 and "radix_fused" in kinds
+    evo.set_wait_limit(1)
+    try:
+        sort()
+        with pytest.raises(evo.EvoSortError) as ei:
+            evo.sync()
+        assert ei.value.status == "ERR_TIMEOUT"
+    finally:
+        evo.set_wait_limit(0)
+    evo.sync()   # the status word was cleared when it was reported
+    check(evo, x, algo="radix")
