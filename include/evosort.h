@@ -139,7 +139,8 @@ typedef struct {
                                  (a call that also names no scratch and no
                                  parameter of the radix kernels: 8192, and 15360
                                  32-bit keys without values);
-                                 1 = off; 2..8192 = that cut-over, whatever the
+                                 1 = off; 2..8192, or 15360 for 32-bit keys
+                                 without values = that cut-over, whatever the
                                  algo */
     long long seg_giant;      /* segmented sort: segments longer than this many
                                  keys are sorted one by one by the device-wide
@@ -167,10 +168,15 @@ size_t evosort_workspace_bytes(size_t n, evosort_dtype dt, int with_values,
  * would run with under params p (NULL = defaults), every default resolved:
  * algorithm, pass kernel, tile shape (with n known the default tile follows
  * the closed form fitted to the tuned tables over log10 n, guarded so that
- * small inputs still give half of the SMs a tile), ranking, thresholds.  The
- * dispatcher's table is not consulted (that needs the keys: evosort_plan), and
- * neither are the decisions taken from the data (the few-values and ordered
- * paths, range reduction).  Host only.  The paper has no counterpart: its
+ * small inputs still give half of the SMs a tile), ranking, thresholds, and
+ * the small-array cut-over that decides at this n.  The tile and ranking are
+ * those of the chain of radix passes: a sort that names them takes that chain,
+ * where one that names nothing may take the one-launch radix sort or the
+ * partition sort (evosort_sort), which have no parameters.  The dispatcher's
+ * table is not consulted (that needs the keys: evosort_plan; a table that names
+ * the mergesort for dt keeps the cut-over at 4096), and neither are the
+ * decisions taken from the data (the few-values and ordered paths, range
+ * reduction).  Host only.  The paper has no counterpart: its
  * parameters are the GA genome of Section 4.2, fixed per run. */
 evosort_status evosort_resolve(size_t n, evosort_dtype dt, int with_values, const evosort_params* p,
                                evosort_params* out);

@@ -547,8 +547,10 @@ static int resolve(const evosort_params* p, int dt, bool pairs, Plan* pl, std::s
         return EVOSORT_ERR_INVALID;
     }
     if (p->small_cap) pl->small_cap = p->small_cap;
-    if (pl->small_cap < 1 || pl->small_cap > kSmallMax) {
-        *err = "params.small_cap must be 0 (default), 1 (off) or at most 8192";
+    // (the dispatcher's own cut-over can be named, so that what evosort_resolve
+    // reports can be passed back)
+    if (pl->small_cap < 1 || (pl->small_cap > kSmallMax && (size_t)pl->small_cap != small_auto_keys(w, pairs))) {
+        *err = "params.small_cap must be 0 (default), 1 (off), at most 8192, or 15360 (32-bit keys without values)";
         return EVOSORT_ERR_INVALID;
     }
     if (p->seg_giant) pl->seg_giant = p->seg_giant;
@@ -613,6 +615,23 @@ static evosort_status finish(int rc, const std::string& err) {
     return (evosort_status)rc;
 }
 
+// The parameters of the radix kernels that a call names: the pass kernels are
+// then the caller's choice.
+static bool names_genes(const evosort_params* p) {
+    return p && (p->keys_per_thread || p->block_size || p->rank_mode || p->pass_kernel || p->adapt_later ||
+                 p->adapt_first);
+}
+
+// Whether one CTA takes arrays above kSmallDefault keys too, up to
+// small_auto_keys: where the call names neither an algorithm, a cut-over,
+// scratch nor a parameter of the radix kernels, and no table may ask for the
+// mergesort.
+static bool small_by_default(const evosort_params* p, int dt) {
+    if (p && (p->algo != EVOSORT_ALGO_AUTO || p->small_cap || p->digit_bits || p->workspace || names_genes(p)))
+        return false;
+    return !table_nonempty() || !table_has_algo(dt, EVOSORT_ALGO_MERGE);
+}
+
 static evosort_status sort_common(const void* in, void* out, const uint32_t* vin, uint32_t* vout, size_t n,
                                   evosort_dtype dt, const evosort_params* p) {
     std::string err;
@@ -656,8 +675,7 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
     evosort_params planned;
     int hybrid = HYBRID_OFF;
     const bool automatic = !p || p->algo == EVOSORT_ALGO_AUTO;
-    const bool own_genes = p && (p->keys_per_thread || p->block_size || p->rank_mode || p->pass_kernel ||
-                                 p->adapt_later || p->adapt_first);   // the pass kernels are the caller's choice
+    const bool own_genes = names_genes(p);
     if (automatic && !own_genes && !(p && p->digit_bits) && n >= kHybridMinAsync) hybrid = HYBRID_ASYNC;
     bool fused = !own_genes;
     // below kDictMinKeys the class only picks a tile, which the one-launch sort
@@ -670,8 +688,7 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
         return cudaStreamIsCapturing(p ? (cudaStream_t)p->stream : nullptr, &cap) == cudaSuccess &&
                cap == cudaStreamCaptureStatusNone;
     };
-    if (automatic && fused && !(p && (p->small_cap || p->digit_bits || p->workspace)) && n <= small_auto_keys(w, pairs) &&
-        (!table_nonempty() || needs_no_sample())) {
+    if (small_by_default(p, dt) && n <= small_auto_keys(w, pairs) && (!table_nonempty() || needs_no_sample())) {
         // one CTA's bins are still done before the one-launch radix sort's
         // barriers over the grid
         Plan sp;
@@ -817,8 +834,11 @@ evosort_status evosort_resolve(size_t n, evosort_dtype dt, int with_values, cons
     out->adapt_first = pl.adapt_first;
     out->seg_warp_cap = pl.seg_warp_cap;
     // the one-CTA path is considered only when the choice is left to the
-    // dispatcher or a cut-over is given (sort_common); otherwise it is off
+    // dispatcher or a cut-over is given (sort_common); otherwise it is off.
+    // Above the default cut-over a second one decides where nothing is named.
     out->small_cap = (p && p->algo != EVOSORT_ALGO_AUTO && p->small_cap <= 1) ? 1 : pl.small_cap;
+    if (n > (size_t)kSmallDefault && small_by_default(p, dt))
+        out->small_cap = (int)small_auto_keys(dtype_bytes(dt), with_values != 0);
     out->seg_giant = pl.seg_giant;
     if (p) {
         out->stream = p->stream;

@@ -243,3 +243,35 @@ def test_binding_wants_tensors_on_the_current_device(monkeypatch):
     with pytest.raises(ValueError, match="CUDA device"):
         evo._need_cuda(_FakeTensor(1, cuda=False))
     evo._need_cuda(None)
+
+
+def test_resolve_reports_the_cut_over_of_calls_that_name_nothing(tmp_path):
+    """Above 4,096 keys a sort that names nothing goes to one CTA up to 8,192
+    keys, or 15,360 of 32 bits without values; resolve says so, takes its own
+    answer back, and says 4096 where the call names scratch, a digit width or a
+    tile, or a table may ask for the mergesort."""
+    import torch
+    import paper_2505_18681_gb300 as evo
+    evo.table_clear()
+    for dtype, pairs, cap in ((torch.int32, False, 15360), (torch.float32, False, 15360), (torch.uint32, True, 8192),
+                              (torch.int64, False, 8192), (torch.float64, True, 8192)):
+        for n in (4097, cap, cap + 1):
+            got = evo.resolve(n, dtype, with_values=pairs)["small_cap"]
+            assert got == cap == evo.resolve(n, dtype, with_values=pairs, algo="auto")["small_cap"]
+            assert evo.resolve(n, dtype, with_values=pairs, algo="radix", small_cap=got)["small_cap"] == cap
+        assert evo.resolve(4096, dtype, with_values=pairs)["small_cap"] == 4096
+    for kw in ({"digit_bits": 8}, {"rank_mode": 3}, {"block_size": 512, "keys_per_thread": 16}, {"small_cap": 4096}):
+        assert evo.resolve(10_000, torch.int32, algo="auto", **kw)["small_cap"] == 4096, kw
+    assert evo.resolve(10_000, torch.int32, algo="radix")["small_cap"] == 1
+    for dtype, pairs, cap in ((torch.int64, False, 15360), (torch.int32, True, 15360), (torch.int32, False, 15361),
+                              (torch.int32, False, 9000)):
+        with pytest.raises(evo.EvoSortError):
+            evo.resolve(10_000, dtype, with_values=pairs, small_cap=cap)
+    t = tmp_path / "t.txt"
+    t.write_text("0 14 0 1 8 0 0 0 32 0 1.0\n")   # int32: mergesort
+    evo.table_load(str(t))
+    try:
+        assert evo.resolve(10_000, torch.int32)["small_cap"] == 4096
+        assert evo.resolve(10_000, torch.int64)["small_cap"] == 8192
+    finally:
+        evo.table_clear()

@@ -112,3 +112,19 @@ def test_bad_cut_over_rejected(evo):
     with pytest.raises(evo.EvoSortError) as ei:
         evo.sort(x, small_cap=9000)
     assert ei.value.status == "ERR_INVALID"
+
+
+@pytest.mark.parametrize("dtype,n", [(torch.int32, 4097), (torch.int32, 15360), (torch.int64, 8192), (torch.int32, 900)],
+                         ids=str)
+def test_resolved_parameters_take_the_same_path(evo, dtype, n):
+    """A sort with what evosort_resolve reports is one launch where the sort
+    that names nothing is."""
+    x = gen(n, dtype, seed=5)
+    got = {k: v for k, v in evo.resolve(n, dtype).items() if k not in ("workspace", "workspace_bytes", "stream")}
+    for kw in ({}, got):
+        y = torch.empty_like(x)
+        k0 = evo.kernel_launches()
+        evo.sort(x, out=y, **kw)
+        evo.sync()
+        assert evo.kernel_launches() - k0 == 1, kw
+        assert np.array_equal(y.cpu().numpy(), oracle.radix_sort(x.cpu().numpy()))
