@@ -680,9 +680,12 @@ static evosort_status sort_common(const void* in, void* out, const uint32_t* vin
     bool fused = !own_genes;
     // below kDictMinKeys the class only picks a tile, which the one-launch sort
     // does not use (unless the table may pick the mergesort): no sample then.
-    // (While a stream is captured the sample stays, and refuses the call.)
+    // (While a stream is captured the sample stays, and refuses the call.  A
+    // caller's digit width other than 8 gives way to the table's, which needs
+    // the class.)
     auto needs_no_sample = [&]() {
         if (!fused || n >= kDictMinKeys || n > fused_max_keys(w, pairs) || n <= kFusedMin) return false;
+        if (p && p->digit_bits && p->digit_bits != 8) return false;
         if (table_has_algo(dt, EVOSORT_ALGO_MERGE)) return false;
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         return cudaStreamIsCapturing(p ? (cudaStream_t)p->stream : nullptr, &cap) == cudaSuccess &&

@@ -179,3 +179,20 @@ def test_barrier_wait_times_out_and_recovers(evo, dtype, n, pairs):
         evo.set_wait_limit(0)
     evo.sync()   # the status word was cleared when it was reported
     check(evo, x, algo="radix")
+
+
+def test_a_named_digit_width_gives_way_to_the_table(evo):
+    """With a table loaded an AUTO sort takes the table's digits whatever width
+    the call names, below the size of the data-dependent paths too."""
+    import os
+    tuned = os.path.join(os.path.dirname(evo.__file__), "tuned", "gb300_int32.txt")
+    x = gen("uniform", 30_000, torch.int32)
+    want = bits(oracle.radix_sort(host(x)))
+    y = torch.empty_like(x)
+    evo.table_load(tuned)
+    for d in (4, 8, 11):
+        assert "radix_fused" in launches(evo, lambda: evo.sort(x, out=y, digit_bits=d))[1], d
+        assert np.array_equal(bits(y), want)
+    evo.table_clear()
+    assert "radix_fused" not in launches(evo, lambda: evo.sort(x, out=y, digit_bits=4))[1]
+    assert np.array_equal(bits(y), want)
