@@ -495,7 +495,8 @@ typedef enum {
     EVOSORT_K_ORDERED = 10,          /* input in order: checked copy (pass 0), check (1), reversed copy (2) */
     EVOSORT_K_RADIX_COUNT = 11,      /* narrow key range: value count and fill (both launches in one record) */
     EVOSORT_K_HYBRID = 12,           /* partition sort of a large array: sample (pass 0), count, plan, step A (3),
-                                        count, scan, step B (6), groups, local sorts (8), clean-up */
+                                        count, scan, step B (6), groups, local sorts (8), clean-up; steps 6 to 8
+                                        run only if the counts did not refuse the keys */
     EVOSORT_K_RADIX_FUSED = 13       /* radix sort of a mid-sized array in one launch; records of the passes
                                         (and the copy) inside it follow, without a time of their own */
 } evosort_kernel_kind;

@@ -312,6 +312,9 @@ int radix_sort(const void* in, void* out, const uint32_t* vin, uint32_t* vout, s
                 return EVOSORT_ERR_CUDA;
             }
             e = cudaMemsetAsync(base, 0, L.zero_end, s);
+            static_assert(PART_GIVEN_UP < 256, "written as the word's lowest byte");
+            if (e == cudaSuccess && call >= 0 && said[HYB_ON])   // for the profile's records
+                e = cudaMemsetAsync(&a.desc[L.npass].hybrid, PART_GIVEN_UP, 1, s);
         }
     }
     const int sms = sm_count();
@@ -1014,8 +1017,11 @@ size_t evosort_profile_read(evosort_kernel_record* out, size_t cap) {
             }
             if (r.kind == EVOSORT_K_RADIX_FIXUP && r.pass >= 0 && r.pass < c.ndesc)
                 active = c.host_desc[r.pass].fixup != FIX_NONE;
-            if (r.kind == EVOSORT_K_HYBRID) active = c.host_desc[c.ndesc - 1].hybrid;
-            if (r.kind == EVOSORT_K_RADIX_HISTOGRAM && c.host_desc[c.ndesc - 1].hybrid) active = 0;
+            const int part = c.host_desc[c.ndesc - 1].hybrid;
+            // given up: all but the steps between the verdict and the clean-up
+            if (r.kind == EVOSORT_K_HYBRID)
+                active = part == PART_DONE || (part == PART_GIVEN_UP && (r.pass < 6 || r.pass == 9));
+            if (r.kind == EVOSORT_K_RADIX_HISTOGRAM && part == PART_DONE) active = 0;
         }
         if (out && k < cap) {
             out[k].kind = r.kind;

@@ -1089,10 +1089,11 @@ __global__ void __launch_bounds__(kHybThreads, 2) hybrid_local(HybArgs a) {
 __global__ void hybrid_finish(HybArgs a) {
     chain_wait();
     if (hyb_on(a.ctl)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) a.last->hybrid = 1;   // for the profile's records
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.last->hybrid = PART_DONE;   // for the profile's records
         return;
     }
     if (a.ctl[HYB_ON] == 0u) return;   // refused by the sample, which writes nothing then
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.last->hybrid = PART_GIVEN_UP;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.scratch16; i += stride)
         ((uint4*)a.scratch)[i] = make_uint4(0u, 0u, 0u, 0u);

@@ -39,6 +39,10 @@ enum : int { ORD_DESCENT = 0, ORD_ASCENT = 1, ORD_EQUAL = 2 };
 enum : int { RNG_NOTMIN = 0, RNG_MAX = 1, RNG_BIAS = 2, RNG_FLAGS = 3, RNG_WORDS = 4 };
 enum : unsigned { RNG_RECORDED = 1u, RNG_REBASED = 2u };
 
+// The partition sort (hybrid.cu): not tried or refused by its sample; sorted
+// the array; given up after its counts.
+enum : int { PART_NONE = 0, PART_DONE = 1, PART_GIVEN_UP = 2 };
+
 struct PassDesc {
     int active;   // 0: the digit is constant over all keys, pass skipped
     int src, dst; // buffer selectors
@@ -46,7 +50,7 @@ struct PassDesc {
     int xout;     // apply from_ordered on store (last active pass)
     int fixup;    // used in the entry after the last pass
     int rank;     // adaptive ranking: the rank mode this pass runs with
-    int hybrid;   // used in the entry after the last pass: the partition sort sorted the array
+    int hybrid;   // used in the entry after the last pass: how far the partition sort came (PART_*)
 };
 
 struct RadixArgs {
@@ -469,6 +473,7 @@ static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int 
     if (threadIdx.x == 0) {
         int active[64];
         int e = 0;
+        const int part = a.desc[a.npass].hybrid;
         // already in order: no pass runs, the input is copied (or, in place,
         // left as it is); in exactly reverse order (for key/value sorts with
         // no two equal keys, so the result stays stable): a reversed copy
@@ -479,6 +484,7 @@ static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int 
                 PassDesc z = {};
                 a.desc[p] = z;
             }
+            a.desc[a.npass].hybrid = part;
             a.desc[a.npass].fixup = reversed ? FIX_REVERSE : (inplace ? FIX_NONE : FIX_IN_TO_OUT);
             return;
         }
@@ -506,6 +512,7 @@ static __global__ void __launch_bounds__(1024) radix_scan_plan(RadixArgs a, int 
         int fix = FIX_NONE;
         if (e == 0 && !inplace) fix = FIX_IN_TO_OUT;
         if (inplace && (e % 2 == 1)) fix = FIX_TMP_TO_OUT;
+        a.desc[a.npass].hybrid = part;
         a.desc[a.npass].fixup = fix;
     }
 }

@@ -160,6 +160,42 @@ def test_captured_graph_decides_anew_for_new_keys(evo):
         assert np.array_equal(bits(y), bits(oracle.radix_sort(host(x)))), name
 
 
+def verdict(evo, fn):
+    """"sorted" by the partition sort, "given up" after its counts, or "refused"
+    by its sample (or not tried), with the radix passes where they had to run."""
+    evo.sync()
+    evo.profile(True)
+    fn()
+    evo.sync()
+    recs = evo.profile_read()
+    evo.profile(False)
+    steps = {r["pass"] for r in recs if r["kind"] == "hybrid" and r["active"]}
+    passes = any(r["kind"] == "radix_onesweep" and r["active"] for r in recs)
+    got = {frozenset(range(10)): "sorted", frozenset(range(6)) | {9}: "given up", frozenset(): "refused"}[frozenset(steps)]
+    assert passes == (got != "sorted")
+    return got
+
+
+VERDICTS = [("uniform", torch.int32, "sorted"), ("uniform", torch.float64, "sorted"), ("float_mix", torch.float64, "sorted"),
+            ("zipf", torch.int64, "refused"), ("gaussian", torch.int64, "refused"),
+            ("paper_exponential", torch.int32, "refused"), ("outliers", torch.int64, "sorted"),
+            ("crowded", torch.int64, "refused"), ("pressed", torch.int64, "given up"), ("frequent", torch.int64, "refused"),
+            ("powers", torch.int64, "refused"), ("powers", torch.float64, "refused")]
+
+
+@pytest.mark.parametrize("table", [False, True], ids=["async", "table"])
+@pytest.mark.parametrize("name,dtype,expect", VERDICTS, ids=lambda v: str(v))
+def test_verdict(evo, name, dtype, expect, table):
+    """How far each kind of keys gets, the same whether the verdict is read back or not."""
+    x = gen(name, N, dtype)
+    if table:
+        for t in TABLES:
+            evo.table_load(t)
+    y = torch.empty_like(x)
+    assert verdict(evo, lambda: evo.sort(x, out=y)) == expect
+    assert np.array_equal(bits(y), bits(oracle.radix_sort(host(x))))
+
+
 @pytest.mark.parametrize("table", [False, True], ids=["async", "table"])
 @pytest.mark.parametrize("dtype", [torch.int64, torch.uint64], ids=str)
 def test_given_up_after_the_counts(evo, dtype, table):
@@ -173,7 +209,7 @@ def test_given_up_after_the_counts(evo, dtype, table):
             evo.table_load(t)
     y, z = torch.empty_like(x), x.clone()
     for _ in range(3):
-        assert taken(evo, lambda: evo.sort(x, out=y)) == (False, True)
+        assert verdict(evo, lambda: evo.sort(x, out=y)) == "given up"
         assert np.array_equal(bits(y), want)
         y.zero_()
     evo.sort(z)
