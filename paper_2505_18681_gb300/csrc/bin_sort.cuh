@@ -19,9 +19,11 @@
 // 7.3 ms with 10,240 32-bit counters.
 //
 // Where the stretches do not separate the keys (a bin of 16 keys or more),
-// the caller's own way (OWN) or block_bin_sort_wide takes over: 32-bit counters, bins of up to 32 *
-// kBinWarpKeys keys sorted by one warp each (bitonic), and if some bin is larger
-// still the merge sort of Algorithm 3, so any input is sorted in bounded time.
+// the caller's own way (OWN) or block_bin_sort_wide takes over: 32-bit counters,
+// bins of equal keys left as they are, others of up to 32 * kBinWarpKeys keys
+// sorted by one warp each (bitonic), and if some bin is longer still, or the
+// keys crowd together from the start, bitonic runs and the merge rounds of
+// Algorithm 3, so any input is sorted in bounded time.
 #pragma once
 
 #include <cfloat>
@@ -34,6 +36,7 @@ namespace evosort {
 constexpr int kBinMax = 1 << 16;     // most bins
 constexpr int kBinThreadKeys = 31;   // longest bin one thread sorts (2^k - 1)
 constexpr int kBinWarpKeys = 16;     // keys per lane of the warp sort
+constexpr int kBinOdd = 32;          // keys beside the frequent one of a longer bin
 
 // Bytes of the second buffer of n keys: the words of the bins, or the merge
 // sort's other array.
@@ -113,6 +116,7 @@ struct XorMap {
     U c;
     __device__ __forceinline__ explicit XorMap(const KeyMap& m) : c((U)(m.s ^ m.x)) {}
     __device__ __forceinline__ U operator()(U k) const { return k ^ c; }
+    __device__ __forceinline__ U forward(U k) const { return k ^ c; }   // the map of the load
 };
 template <typename U>
 struct FloatIn {
@@ -126,6 +130,7 @@ struct GeneralOut {   // any key type
     KeyMap m;
     __device__ __forceinline__ explicit GeneralOut(const KeyMap& k) : m(k) {}
     __device__ __forceinline__ U operator()(U k) const { return map_inv(k, m); }
+    __device__ __forceinline__ U forward(U k) const { return map_fwd(k, m); }
 };
 template <typename U>
 struct FloatOut : GeneralOut<U> {
@@ -203,9 +208,9 @@ __device__ __forceinline__ ValuePosition<U, MO> block_value_position(const U (&k
 
 template <typename U, int NT>
 struct BinShared {
-    U mn[NT / 32], mx[NT / 32];
+    U mn[NT / 32], mx[NT / 32];   // extents; later the keys of a long bin that are not its frequent one
     uint32_t wsum[NT / 32 + 1];
-    uint32_t nlist, big;
+    uint32_t nlist, nodd;
     uint32_t list[512];   // bins left to the warps: first position | length << 16
 };
 
@@ -295,10 +300,7 @@ __device__ __noinline__ void bin_warp_sort(U* k, int c) {
     const int lane = threadIdx.x & 31;
     U x[kBinWarpKeys];
 #pragma unroll
-    for (int r = 0; r < kBinWarpKeys; ++r) {
-        const int i = lane * kBinWarpKeys + r;
-        x[r] = i < c ? k[i] : ~(U)0;
-    }
+    for (int r = 0; r < kBinWarpKeys; ++r) x[r] = r * 32 + lane < c ? k[r * 32 + lane] : ~(U)0;
     warp_bitonic_sort<U, kBinWarpKeys>(x);
     __syncwarp();
 #pragma unroll
@@ -308,37 +310,103 @@ __device__ __noinline__ void bin_warp_sort(U* k, int c) {
     }
 }
 
+// Sort of k[0..m) by the CTA if all but kBinOdd of the keys are one value: the
+// others go around it.  False, and nothing moved, if they are not.
+template <typename U, int NT>
+__device__ __forceinline__ bool bin_one_value(U* k, int m, BinShared<U, NT>& sh) {
+    static_assert(kBinOdd <= 2 * (NT / 32), "room of the extents");
+    const int tid = threadIdx.x;
+    U* const odds = sh.mn;   // (mx lies behind it)
+    const U a = k[0], b = k[m / 2], c = k[m - 1];
+    const U most = a == b || a == c ? a : b;
+    if (tid == 0) sh.nodd = 0u;
+    __syncthreads();
+    for (int i = tid; i < m; i += NT) {
+        const U x = k[i];
+        if (x != most) {
+            const uint32_t at = atomicAdd(&sh.nodd, 1u);
+            if (at < (uint32_t)kBinOdd) odds[at] = x;
+        }
+    }
+    __syncthreads();
+    const int odd = (int)sh.nodd;
+    if (odd > kBinOdd) return false;
+    if (odd > 0) {
+        int less = 0;
+        for (int i = 0; i < odd; ++i) less += odds[i] < most;
+        for (int i = tid; i < m - odd; i += NT) k[less + i] = most;
+        if (tid < odd) {
+            const U x = odds[tid];
+            int rank = 0;
+            for (int i = 0; i < odd; ++i) rank += odds[i] < x || (odds[i] == x && i < tid);
+            k[x < most ? rank : m - odd + rank] = x;
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
 // The keys of k0 stand in their bins (starts in k1, ends of a thread's last
 // bin in run, multi: its bins of two or more keys): sorts the bins, the long
 // ones (heavy: there are some) by a warp each, or everything if some bin is
-// longer still.
+// longer still and holds several frequent values.
 template <typename U, int NT, int BPT>
 __device__ __forceinline__ const U* bin_finish(U* k0, U* k1, int n, uint32_t multi, uint32_t run, bool heavy,
                                                BinShared<U, NT>& sh) {
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t* const own = (const uint32_t*)k1 + tid * BPT;
-    if (tid == 0) sh.nlist = sh.big = 0u;
+    if (tid == 0) sh.nlist = 0u;
     __syncthreads();
     while (multi) {
         const int q = __ffs((int)multi) - 1;
         multi &= multi - 1u;
         const uint32_t at = own[q], next = q + 1 < BPT ? own[q + 1] : run;
         const int m = (int)(next - at);
-        if (m <= kBinThreadKeys) {
+        if (m <= kBinThreadKeys)
             bin_insertion(k0 + at, m);
-        } else if (m <= 32 * kBinWarpKeys) {
+        else
             sh.list[atomicAdd(&sh.nlist, 1u)] = at | (uint32_t)m << 16;   // n / (kBinThreadKeys + 1) entries at most
-        } else {
-            sh.big = 1u;
-        }
     }
     __syncthreads();
     if (!heavy) return k0;
-    if (sh.big) return smem_merge_sort<U, false, 8>(k0, k1, nullptr, nullptr, n, 8) ? k1 : k0;
-    const int m = (int)sh.nlist;
-    for (int e = warp; e < m; e += NT / 32) bin_warp_sort(k0 + (sh.list[e] & 0xFFFFu), (int)(sh.list[e] >> 16));
+    const int listed = (int)sh.nlist;
+    for (int e = 0; e < listed; ++e) {
+        const int m = (int)(sh.list[e] >> 16);
+        if (m > 32 * kBinWarpKeys && !bin_one_value<U, NT>(k0 + (sh.list[e] & 0xFFFFu), m, sh))
+            return smem_sort_any(k0, k1, n);   // (k1's starts are not needed any more)
+    }
+    for (int e = warp; e < listed; e += NT / 32) {
+        U* const k = k0 + (sh.list[e] & 0xFFFFu);
+        const int m = (int)(sh.list[e] >> 16);
+        if (m > 32 * kBinWarpKeys) continue;
+        const U first = k[0];
+        bool other = false;
+        for (int i = lane; i < m; i += 32) other |= k[i] != first;
+        if (__any_sync(0xffffffffu, other)) bin_warp_sort(k, m);
+    }
     __syncthreads();
     return k0;
+}
+
+// What the keys of a warp say of all: x is a sampled key of each lane that
+// have()s one, from all over the array.  near: lanes whose key shares a 1024th of
+// the range; a lane's key is compared with the first of them.
+struct KeyVotes {
+    bool crowded, repeated, frequent;   // another key there; the same key; and a third of the warp with it
+};
+template <typename U, typename P>
+__device__ __forceinline__ KeyVotes key_votes(U x, bool have, const P& position) {
+    const uint32_t some = __ballot_sync(0xffffffffu, have);
+    KeyVotes v = {false, false, false};
+    if (have) {
+        const uint32_t near = __match_any_sync(some, position(x) >> 22);
+        const int first = __ffs((int)near) - 1;
+        const bool same = __shfl_sync(near, x, first) == x;
+        v.crowded = !same;
+        v.repeated = same && first != (int)(threadIdx.x & 31);
+        v.frequent = same && __popc(near) >= 10;
+    }
+    return v;
 }
 
 template <int NT, int BPT, typename U>
@@ -348,15 +416,58 @@ __device__ __forceinline__ void bin_zero(U* k1) {
     for (int j = 0; j < BPT / 4; ++j) mine[j] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// The position as block_bin_sort_wide is given it: one of the keys' range is
+// made from the range (as an argument its registers cost 1.5 % of 10,000 segments
+// of int32 keys, which never need it).
+template <typename P>
+struct WidePosition {
+    P p;
+    __device__ __forceinline__ explicit WidePosition(const P& position) : p(position) {}
+    template <typename U>
+    __device__ __forceinline__ P get(U, unsigned long long) const { return p; }
+};
+template <typename U>
+struct WidePosition<KeyPosition<U>> {
+    __device__ __forceinline__ WidePosition() {}
+    __device__ __forceinline__ explicit WidePosition(const KeyPosition<U>&) {}
+    __device__ __forceinline__ KeyPosition<U> get(U lo, unsigned long long width) const {
+        return {lo, __clzll((long long)(width | 1ull))};
+    }
+};
+
 // The same sort with 32-bit counters and any distribution of the keys, which
 // lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per
-// thread: the words of block_bin_sort, so that k1 is as large as there.
-template <typename U, int NT, int KPT, int BPT>
-__device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, U* k0, U* k1,
-                                                     BinShared<U, NT>& sh) {
+// thread: the words of block_bin_sort, so that k1 is as large as there.  With
+// ask, one key of each thread tells first whether bins can separate them at all
+// (a quarter of these keys share a 1024th of the range with a different one: they
+// cannot), and whether some value is so frequent that a warp's equal bins are
+// better added up before the counters see them (it costs more where they differ:
+// 2,000 segments of 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose
+// values crowd together are tried once more by their bit patterns, which spread
+// magnitudes evenly.  Bins of one value are left as they are: 1e8 int64 keys with
+// some 40 keys of each value, partition sort, 23.2 -> 3.7 ms (every bin by a warp
+// before, or everything merged).
+template <typename U, int NT, int KPT, int BPT, typename P>
+__device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, WidePosition<P> given,
+                                                     bool ask, U* k0, U* k1, BinShared<U, NT>& sh) {
+    const P position = given.get(lo, width);
     static_assert(BPT % 8 == 4 && BPT * NT <= kBinMax, "bins per thread");
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    bool add_up = false;
+    if (ask) {
+        const int at = lane % ((n + NT - 1) / NT) * NT + tid;
+        const KeyVotes v = key_votes(at < n ? k0[at] : (U)0, at < n, position);
+        const int most = min(n, NT);
+        if (4 * __syncthreads_count(v.crowded) > most) {
+            if constexpr (P::linear)
+                return smem_sort_any(k0, k1, n);
+            else
+                return block_bin_sort_wide<U, NT, KPT, BPT, KeyPosition<U>>(
+                    n, lo, width, WidePosition<KeyPosition<U>>(), true, k0, k1, sh);
+        }
+        add_up = 4 * __syncthreads_count(v.frequent) > most;
+    }
     uint32_t* const bins = (uint32_t*)k1;
     // A thread's BPT bins are consecutive and read four at a time; with BPT / 4
     // odd, a quarter-warp's 16-byte reads fall in different banks.
@@ -366,18 +477,30 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
 #pragma unroll
     for (int i = 0; i < KPT; ++i) key[i] = i * NT + tid < n ? k0[i * NT + tid] : (U)0;
     int lz;
-    uint32_t mult;
-    cut_range(width, (uint32_t)(BPT * NT), &lz, &mult);
+    uint32_t mult = (uint32_t)(BPT * NT);
+    if (P::linear) cut_range(width, (uint32_t)(BPT * NT), &lz, &mult);
+    const uint32_t lt = lanemask_lt();
     __syncthreads();
-    if (tid == 0) sh.nlist = sh.big = 0u;
     // ---- count; the old count is the key's place in its bin
     uint32_t br[KPT];   // bin | place << 16
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-        if (i * NT + tid < n) {
+        const bool have = i * NT + tid < n;
+        const uint32_t some = __ballot_sync(0xffffffffu, have);
+        if (have) {
             // (in range for every key of [lo, lo + width]; never out of the array for any other)
-            const uint32_t b = min(__umulhi(norm32((U)(key[i] - lo), lz), mult), (uint32_t)(BPT * NT - 1));
-            br[i] = b | atomicAdd(&bins[b], 1u) << 16;
+            const uint32_t b = min(__umulhi(position(key[i]), mult), (uint32_t)(BPT * NT - 1));
+            uint32_t place;
+            if (add_up) {
+                const uint32_t peers = __match_any_sync(some, b);
+                const int leader = __ffs((int)peers) - 1;
+                place = 0u;
+                if (lane == leader) place = atomicAdd(&bins[b], (uint32_t)__popc(peers));
+                place = __shfl_sync(peers, place, leader) + (uint32_t)__popc(peers & lt);
+            } else {
+                place = atomicAdd(&bins[b], 1u);
+            }
+            br[i] = b | place << 16;
         }
     }
     __syncthreads();
@@ -416,7 +539,7 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         mine[j] = q;
         run = d;
     }
-    const bool one_value = width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
+    const bool one_value = P::linear && width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
     const bool heavy = __syncthreads_or(!one_value && any > (uint32_t)kBinThreadKeys);
 
     // ---- every key to its place
@@ -522,8 +645,10 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
 #pragma unroll
                 for (int i = 0; i < KPT; ++i)
                     if (i * NT + tid < n) k0[i * NT + tid] = key[i];
-                __syncthreads();
-                const U* r = block_bin_sort_wide<U, NT, KPT, WPT>(n, lo, width, k0, k1, sh);
+                // (bins of fewer than 32 keys: the threads sort them, whatever the keys)
+                const bool mild = !__syncthreads_or((any & 0xE0E0E0E0u) != 0u) && __reduce_add_sync(0xffffffffu, v) == (uint32_t)n;
+                const U* r = block_bin_sort_wide<U, NT, KPT, WPT, P>(n, lo, width, WidePosition<P>(position), !mild, k0,
+                                                                     k1, sh);
                 placed();
                 return r;
             }

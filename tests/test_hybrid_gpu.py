@@ -216,3 +216,21 @@ def test_given_up_after_the_counts(evo, dtype, table):
     evo.sort(x, out=y, descending=True)
     evo.sync()
     assert np.array_equal(bits(z), want) and np.array_equal(bits(y), want[::-1])
+
+
+@pytest.mark.parametrize("copies", [10, 40, 300])
+@pytest.mark.parametrize("dtype", [torch.int32, torch.int64, torch.float64], ids=str)
+def test_repeated_values(evo, dtype, copies):
+    """Some copies of every value, spread over the whole type: more of them than
+    the local sorts' bins count, fewer than the sample takes for frequent."""
+    values = gen("uniform", N // copies, torch.int64)
+    pick = gen("uniform", N, torch.int64, seed=copies).remainder(N // copies)
+    x = values[pick]
+    x = (x >> 32).to(dtype) if dtype == torch.int32 else x.to(dtype)
+    want = bits(oracle.radix_sort(host(x)))
+    y = torch.empty_like(x)
+    assert verdict(evo, lambda: evo.sort(x, out=y)) == "sorted"
+    assert np.array_equal(bits(y), want)
+    evo.sort(x, out=y, descending=True)
+    evo.sync()
+    assert np.array_equal(bits(y), want[::-1])
