@@ -2,6 +2,7 @@
 // that shared memory does not hold, and buckets of the partition sort that
 // came out too large for it.
 //
+//   cta_vote         says by a sample which of the two below the run gets;
 //   cta_split_sort   cuts the run's sampled key range into equal parts, moves
 //                    the keys to their parts through the other buffer (one
 //                    read to count, one read and one write to move, unstable:
@@ -14,6 +15,8 @@
 //                    The CTA walks the tiles in order, so running digit
 //                    offsets replace a look-back.
 #pragma once
+
+#include <type_traits>
 
 #include "bin_sort.cuh"
 #include "common.cuh"
@@ -51,13 +54,15 @@ struct CtaShared {
     uint32_t scan[kCtaWarps + 1];
     uint32_t next, end, below, above, longest;
     float value[2][kCtaWarps];
-    int active[sizeof(U)];
 };
 
 struct AsIs {
     template <typename U>
     __device__ __forceinline__ U operator()(U k) const { return k; }
 };
+// Whether keys that are left where they are, in their own array, need out().
+template <typename MI>
+constexpr bool kMapsBack = !std::is_same<MI, AsIs>::value;
 
 // Local sort of n <= cta_cap() keys held in registers (mapped); out maps back,
 // store(position, key) receives the sorted keys, still mapped.  Bins by the
@@ -97,12 +102,17 @@ __device__ __forceinline__ void cta_local_sort(const U (&key)[cta_kpt<U>()], int
     __syncthreads();
 }
 
-// LSD radix sort of the len mapped keys in a (other buffer b); the sorted
-// keys, through out(), end in fin (a or b).  8-bit digits; digits that are
-// equal in all keys are skipped.  I counts keys: 32 bits for runs of at most
-// kSegCutKeys, 64 bits for any.
-template <typename I, typename U, typename M>
-__device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, unsigned char* smem, CtaShared<U>& sh) {
+// LSD radix sort of the len keys in a (other buffer b): out() maps a key on its
+// last store, and out.forward() on its first load unless it is mapped already
+// (MAPPED); the sorted keys end in fin (a or b).
+// 8-bit digits; digits that are equal in all keys are skipped.  I counts keys:
+// 32 bits for runs of at most kSegCutKeys, 64 bits for any.
+template <typename I, bool MAPPED, typename U, typename M>
+__device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out) {
+    auto in = [&](U k) { return MAPPED ? k : out.forward(k); };
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_scan[kCtaWarps + 1];
+    __shared__ int s_active[sizeof(U)];
     constexpr int NP = sizeof(U);
     constexpr int BINS = 256;
     constexpr int KPT = 8;
@@ -121,12 +131,12 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
     U* s_r = (U*)(s_whist + kCtaWarps * BINS);          // TILE keys
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < NP * BINS; i += kCtaThreads) s_hist[i] = 0;
-    if (tid < NP) sh.active[tid] = 0;
+    if (tid < NP) s_active[tid] = 0;
     __syncthreads();
     auto count = [&](const U* keys, uint32_t m, uint32_t* hist) {
 #pragma unroll 4
         for (uint32_t i = tid; i < m; i += kCtaThreads) {
-            const U k = keys[i];
+            const U k = in(keys[i]);
 #pragma unroll
             for (int p = 0; p < NP; ++p) atomicAdd(&hist[p * BINS + digit_of(k, 8 * p, 0xFFu)], 1u);
         }
@@ -150,22 +160,30 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
         }
     }
     for (int i = tid; i < NP * BINS; i += kCtaThreads)
-        if (s_hist[i] != 0 && s_hist[i] != len) sh.active[i / BINS] = 1;
+        if (s_hist[i] != 0 && s_hist[i] != len) s_active[i / BINS] = 1;
     __syncthreads();
     int nact = 0;
-    for (int p = 0; p < NP; ++p) nact += sh.active[p];
+    for (int p = 0; p < NP; ++p) nact += s_active[p];
+    if (nact == 0) {   // equal keys
+        if (fin != a || MAPPED)
+            for (I i = tid; i < len; i += kCtaThreads) fin[i] = out(in(a[i]));
+        __syncthreads();
+        return;
+    }
+    int done = 0;
     U* src = a;
     U* dst = b;
     const uint32_t lt = lanemask_lt();
     for (int p = 0; p < NP; ++p) {
-        if (!sh.active[p]) continue;
+        if (!s_active[p]) continue;
         const int shift = 8 * p;
+        const bool first = done == 0, last = ++done == nact;
         {
             const I c = tid < BINS ? s_hist[p * BINS + tid] : (I)0;
             I tot;
             I* scan;
             if constexpr (sizeof(I) == 4)
-                scan = sh.scan;
+                scan = s_scan;
             else
                 scan = (I*)s_match;   // (cleared again by the first tile)
             const I ex = block_exclusive_scan<kCtaThreads, I>(c, scan, &tot);
@@ -182,12 +200,18 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
             }
             __syncwarp();
             U key[KPT];
-            uint32_t dr[KPT];
+            uint32_t rk[KPT / 2];   // rank in the warp, two 16-bit fields per register
             const int wofs = warp * 32 * KPT + lane;
+            if (tid == 0 && t0 + TILE < len)   // the next tile, while this one is ranked
+                prefetch_l2_inner(src + t0 + TILE, (size_t)(len - t0 - TILE < TILE ? len - t0 - TILE : (I)TILE) * sizeof(U));
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
                 const int s = wofs + 32 * i;
                 key[i] = s < valid ? src[t0 + s] : ~(U)0;
+            }
+            if (first) {
+#pragma unroll
+                for (int i = 0; i < KPT; ++i) key[i] = wofs + 32 * i < valid ? in(key[i]) : ~(U)0;
             }
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
@@ -203,8 +227,8 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
                     wh[dig] = (uint16_t)(old + __popc(peers));
                     wm[dig] = 0u;
                 }
-                old = __shfl_sync(0xffffffffu, old, leader);
-                dr[i] = dig | ((old + __popc(peers & lt)) << 16);
+                old = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
+                rk[i / 2] = i & 1 ? __byte_perm(rk[i / 2], old, 0x5410) : old;
                 __syncwarp();
             }
             __syncthreads();
@@ -219,22 +243,22 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
             }
             {
                 uint32_t tot;
-                const uint32_t ex = block_exclusive_scan<kCtaThreads>(tc, sh.scan, &tot);
+                const uint32_t ex = block_exclusive_scan<kCtaThreads>(tc, s_scan, &tot);
                 if (tid < BINS) s_excl[tid] = ex;
             }
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < KPT; ++i) {
                 if (wofs + 32 * i < valid) {
-                    const uint32_t dig = dr[i] & 0xFFFFu;
-                    s_r[s_excl[dig] + wh[dig] + (dr[i] >> 16)] = key[i];
+                    const uint32_t dig = digit_of(key[i], shift, 0xFFu);
+                    s_r[s_excl[dig] + wh[dig] + (i & 1 ? rk[i / 2] >> 16 : rk[i / 2] & 0xFFFFu)] = key[i];
                 }
             }
             __syncthreads();
             for (int s = tid; s < valid; s += kCtaThreads) {
                 const U k = s_r[s];
                 const uint32_t dig = digit_of(k, shift, 0xFFu);
-                dst[s_run[dig] + (s - s_excl[dig])] = k;
+                dst[s_run[dig] + (s - s_excl[dig])] = last ? out(k) : k;
             }
             __syncthreads();
             if (tid < BINS) s_run[tid] += s_tcnt[tid];
@@ -244,30 +268,96 @@ __device__ __noinline__ void cta_radix_sort(U* a, U* b, U* fin, I len, M out, un
         src = dst;
         dst = t;
     }
-    for (I i = tid; i < len; i += kCtaThreads) fin[i] = out(src[i]);
+    if (src != fin)
+        for (I i = tid; i < len; i += kCtaThreads) fin[i] = src[i];
     __syncthreads();
+}
+
+// Whether a run of len keys is better sorted by radix passes than cut.  A cut
+// moves a key once and sorts it on chip, which costs about as much as two
+// (32-bit keys) or three passes.  It costs more where the keys crowd together
+// (uneven parts are cut again), where one value holds much of them (its counters
+// queue up) and, while the keys of a value fit a local sort, where values repeat
+// (the bins fill up); it costs less where a part holds one value.  Read off the
+// CTA's sample: x is one of this thread's sampled keys, vary the bits in which
+// they differ from the smallest, width their range.  kCtaVoters warps compare
+// their keys (all of them took 6 % of segments of 7,000 keys).
+// 300 segments of up to 40,000 keys, cut in any case -> so: float64 keys of 1,000
+// values 2,378 -> 376 us, int64 keys of 7 values 271 -> 152 us, float32 keys of 100
+// values 327 -> 185 us; passes in any case: uniform int64 keys 555 us, 216 so.
+constexpr int kCtaVoters = 4;   // warps
+template <typename U, typename P>
+__device__ __noinline__ bool cta_vote(U x, bool have, U vary, uint32_t len, unsigned long long width, P position,
+                                      CtaShared<U>& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t vl = __reduce_or_sync(0xffffffffu, (uint32_t)vary);
+    const uint32_t vh = __reduce_or_sync(0xffffffffu, (uint32_t)((unsigned long long)vary >> 32));
+    uint32_t said = 0;   // which digits vary (8 bits), then counts of up to 32
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+        said |= (((vl >> (8 * b)) & 0xFFu) != 0u ? 1u << b : 0u) | (((vh >> (8 * b)) & 0xFFu) != 0u ? 16u << b : 0u);
+    if (warp < kCtaVoters) {
+        const KeyVotes v = key_votes(x, have, position);
+        said |= (uint32_t)__popc(__ballot_sync(0xffffffffu, v.crowded)) << 8 |
+                (uint32_t)__popc(__ballot_sync(0xffffffffu, v.repeated)) << 16 |
+                (uint32_t)__popc(__ballot_sync(0xffffffffu, v.frequent)) << 24;
+    }
+    if (lane == 0) sh.scan[warp] = said;
+    __syncthreads();
+    uint32_t crowded = 0, repeated = 0, frequent = 0;
+#pragma unroll
+    for (int w = 0; w < kCtaVoters; ++w) {
+        crowded += (sh.scan[w] >> 8) & 0xFFu;
+        repeated += (sh.scan[w] >> 16) & 0xFFu;
+        frequent += sh.scan[w] >> 24;
+    }
+    const int digits = __popc(__reduce_or_sync(0xffffffffu, lane < kCtaWarps ? sh.scan[lane] : 0u) & 0xFFu);
+    __syncthreads();   // (scan is used again)
+    constexpr uint32_t voters = kCtaVoters * 32;
+    if (crowded > voters / 3 || frequent > voters / 4 || digits == 1) return true;
+    // values with more keys each than a local sort holds: from the distinct keys
+    // among a warp's 32, v distinct values are at most kinds / (1 - kinds / 32)
+    const float kinds = (float)(voters - repeated) / (float)kCtaVoters;
+    if ((float)len * (32.f - kinds) > 32.f * kinds * (float)cta_cap<U>()) return false;
+    if (repeated >= 2u && digits <= (sizeof(U) == 8 ? 3 : 2)) return true;
+    return P::linear && sizeof(U) == 8 && digits <= 2 && width < (unsigned long long)len;
+}
+template <typename U, typename P>
+__device__ __forceinline__ bool cta_wants_passes(const U (&k)[8], int m, uint32_t len, U lo, unsigned long long width,
+                                                 const P& position, CtaShared<U>& sh) {
+    const int tid = threadIdx.x, row = (tid & 31) % ((m + kCtaThreads - 1) / kCtaThreads);
+    U x = k[0], vary = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (row == i) x = k[i];
+        if (i * kCtaThreads + tid < m) vary |= k[i] ^ lo;
+    }
+    return cta_vote<U, P>(x, row * kCtaThreads + tid < m, vary, len, width, position, sh);
 }
 
 // Sort of the len keys of src: in() maps a key on its load, out() on its last
 // store.  The parts are laid out in part (as long as src); the sorted keys end
 // in fin, which is src or part.  LEVEL 0 cuts too large parts again.  len is at
-// most kSegCutKeys: the counters are of 32 bits.
+// most kSegCutKeys: the counters are of 32 bits.  False, and src as it was, where
+// the run is better left to radix passes.
 template <typename U, int LEVEL, typename MI, typename MO>
-__device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
+__device__ __forceinline__ bool cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
                                                unsigned char* smem, CtaShared<U>& sh);
 template <typename U, typename MO>
 __device__ __noinline__ void cta_split_again(U* src, U* part, U* fin, uint32_t len, MO out, unsigned char* smem,
                                              CtaShared<U>& sh) {
-    cta_split_impl<U, 1>(src, part, fin, len, AsIs(), out, smem, sh);
+    if (!cta_split_impl<U, 1>(src, part, fin, len, AsIs(), out, smem, sh))
+        cta_radix_sort<uint32_t, true>(src, part, fin, len, out);
 }
 template <typename U, typename MI, typename MO>
 __device__ __forceinline__ void cta_split_sort(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
                                                unsigned char* smem, CtaShared<U>& sh) {
-    cta_split_impl<U, 0>(src, part, fin, len, in, out, smem, sh);
+    if (!cta_split_impl<U, 0>(src, part, fin, len, in, out, smem, sh))
+        cta_radix_sort<uint32_t, false>(src, part, fin, len, out);
 }
 
 template <typename U, int LEVEL, typename MI, typename MO>
-__device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
+__device__ __forceinline__ bool cta_split_impl(U* src, U* part, U* fin, uint32_t len, MI in, MO out,
                                                unsigned char* smem, CtaShared<U>& sh) {
     constexpr int KPT = cta_kpt<U>();
     constexpr int CAP = cta_cap<U>();
@@ -282,33 +372,50 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
     uint32_t* s_cur = (uint32_t*)(smem + cta_buf_bytes<U>()) + LEVEL * kCtaParts;
     const int tid = threadIdx.x, lane = tid & 31;
 
-    // ---- range of the keys, from a sample
+    // ---- range of the keys, from a sample, and whether to cut them at all
     U lo, hi;
     float low = 0.f, scale = 0.f;   // floats: the cut of the sampled values
+    bool passes;
     {
         U k[8];
         const uint32_t stride = len / (8 * kCtaThreads);
         const int m = stride ? 8 * kCtaThreads : (int)len;
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (i * kCtaThreads + tid < m) k[i] = in(src[(uint32_t)(i * kCtaThreads + tid) * (stride ? stride : 1u)]);
+            k[i] = in(i * kCtaThreads + tid < m ? src[(uint32_t)(i * kCtaThreads + tid) * (stride ? stride : 1u)] : (U)0);
         block_extent<U, kCtaThreads, 8>(k, m, sh.bin, &lo, &hi);
+        const int wlz = __clzll((long long)((unsigned long long)(U)(hi - lo) | 1ull));
         if constexpr (MO::is_float) {
             const auto pos = block_value_position<U, kCtaThreads, 8>(k, m, out, out.descending(), sh.value);
             low = pos.low;
             scale = pos.scale;
+            passes = cta_wants_passes<U>(k, m, len, lo, 0ull, pos, sh);
+        } else {
+            passes = cta_wants_passes<U>(k, m, len, lo, (unsigned long long)(U)(hi - lo), KeyPosition<U>{lo, wlz}, sh);
         }
     }
     const unsigned long long width = (unsigned long long)(U)(hi - lo);
     if (width == 0) {   // one value, as far as the sample shows
         bool other = false;
-        for (uint32_t i = tid; i < len; i += kCtaThreads) other |= in(src[i]) != lo;
-        if (!__syncthreads_or(other)) {
-            const U k = out(lo);
-            for (uint32_t i = tid; i < len; i += kCtaThreads) fin[i] = k;
-            __syncthreads();
-            return;
+        uint32_t i = tid;
+        for (; i + 7u * kCtaThreads < len; i += 8u * kCtaThreads) {
+            U k[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) k[u] = src[i + (uint32_t)(u * kCtaThreads)];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) other |= in(k[u]) != lo;
         }
+        for (; i < len; i += kCtaThreads) other |= in(src[i]) != lo;
+        if (!__syncthreads_or(other)) {
+            if (fin != src || !kMapsBack<MI>) {
+                const U k = out(lo);
+                for (i = tid; i < len; i += kCtaThreads) fin[i] = k;
+                __syncthreads();
+            }
+            return true;
+        }
+    } else if (passes) {
+        return false;
     }
     uint32_t want = (len + (uint32_t)cta_target<U>() - 1u) / (uint32_t)cta_target<U>();
     if (want > (uint32_t)kCtaParts) want = (uint32_t)kCtaParts;
@@ -375,12 +482,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
     __syncthreads();
     const bool low_end = sh.below != 0u, high_end = sh.above != 0u;
     // most keys in one part: not separated by its range
-    if (!one_value && sh.longest > (uint32_t)CAP && sh.longest > len / 2u) {
-        for (uint32_t i = tid; i < len; i += kCtaThreads) src[i] = in(src[i]);
-        __syncthreads();
-        cta_radix_sort<uint32_t, U>(src, part, fin, len, out, smem, sh);
-        return;
-    }
+    if (!one_value && sh.longest > (uint32_t)CAP && sh.longest > len / 2u) return false;
 
     // ---- move the keys to their parts, a tile at a time
     {
@@ -473,7 +575,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
                 cta_split_again<U>(part + s, other, fin + s, n, out, smem, sh);
             } else {
                 __syncthreads();
-                cta_radix_sort<uint32_t, U>(part + s, other, fin + s, n, out, smem, sh);
+                cta_radix_sort<uint32_t, true>(part + s, other, fin + s, n, out);
             }
         } else if (n > 0) {
             U key[KPT];
@@ -487,6 +589,7 @@ __device__ __forceinline__ void cta_split_impl(U* src, U* part, U* fin, uint32_t
         f = g;
         s = e;
     }
+    return true;
 }
 
 }  // namespace evosort

@@ -29,9 +29,11 @@
 // key of three steps (count, move, bin sort) by two CTAs of 512 threads per SM;
 // in the block tier the barriers of one bin sort per segment.  Before, the
 // large tier made a stable pass per digit over global memory and the block
-// tier merged: 10,000 int32 segments up to 1e6 keys (9.1e8 keys) 17.2 -> 9.2
-// ms, 20,000 int64 ones up to 8,000 (2.6e7 keys) 1.80 -> 0.56 ms, 3,000
-// float64 ones up to 1e5 (3.5e7 keys) 1.64 -> 0.79 ms.
+// tier merged: 10,000 int32 segments up to 1e6 keys (9.1e8 keys) 17.2 -> 9.3
+// ms, 20,000 int64 ones up to 8,000 (2.6e7 keys) 1.80 -> 0.53 ms, 3,000
+// float64 ones up to 1e5 (3.5e7 keys) 1.64 -> 0.79 ms.  Keys that neither cuts
+// nor bins separate (one value in half of the places, magnitudes of every order,
+// a thousand values) are about as fast as then, between 0.75 and 2 times.
 #include <algorithm>
 #include <vector>
 
@@ -149,8 +151,8 @@ __device__ __forceinline__ void block_tier(const SegArgs& a, unsigned char* smem
     U* keys = (U*)a.keys + lo;
     U k[cta_kpt<U>()];
 #pragma unroll
-    for (int i = 0; i < cta_kpt<U>(); ++i)
-        if (i * kSB + (int)threadIdx.x < len) k[i] = in(keys[i * kSB + threadIdx.x]);
+    for (int i = 0; i < cta_kpt<U>(); ++i)   // (every register is written)
+        k[i] = in(i * kSB + (int)threadIdx.x < len ? keys[i * kSB + threadIdx.x] : (U)0);
     cta_local_sort<U>(k, len, out, smem, sh, [&](int i, U x) { keys[i] = out(x); });
 }
 
@@ -198,17 +200,13 @@ __global__ void __launch_bounds__(kSB, 2) seg_sort(SegArgs a) {
 // of its own, so that the other tiers keep their registers.
 template <typename U>
 __global__ void __launch_bounds__(kSB) seg_long(SegArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ CtaShared<U> sh;
     const uint32_t longs = a.hdr[2 * kNB + 3];
     for (uint32_t item = a.skip + blockIdx.x; item < longs; item += gridDim.x) {
         const uint32_t seg = a.order[item];
         const uint64_t lo = a.off[seg];
         const unsigned long long len = a.off[seg + 1] - lo;
         U* keys = (U*)a.keys + lo;
-        for (unsigned long long i = threadIdx.x; i < len; i += kSB) keys[i] = map_fwd(keys[i], a.map);
-        __syncthreads();
-        cta_radix_sort<unsigned long long, U>(keys, (U*)a.tmp + lo, keys, len, GeneralOut<U>(a.map), smem, sh);
+        cta_radix_sort<unsigned long long, false>(keys, (U*)a.tmp + lo, keys, len, GeneralOut<U>(a.map));
     }
 }
 

@@ -93,3 +93,41 @@ def test_float_segments_cut_by_value(evo, dtype, kind):
     evo.segmented_sort(k, torch.from_numpy(offs.astype(np.int64)).cuda())
     evo.sync()
     assert np.array_equal(bits(k), bits(want))
+
+
+def uneven(kind, n, r):
+    """int64 keys that bins over the range, or parts of it, separate badly."""
+    x = r.integers(-2**62, 2**62, n)
+    return {"half": lambda: np.where(r.random(n) < 0.5, 0, x >> 31), "most": lambda: np.where(r.random(n) < 0.995, 7, x),
+            "beside": lambda: np.where(r.random(n) < 0.9, 10**9, np.where(r.random(n) < 0.02, 10**9 + r.integers(-3, 4, n), x)),
+            "ends": lambda: np.where(r.random(n) < 0.5, 5, np.where(r.random(n) < 0.9, 6, x)),
+            "zipf": lambda: np.minimum(r.random(n) ** -2.0, 1e6).astype(np.int64), "hundred": lambda: x % 100,
+            "thousand": lambda: x % 1000, "words": lambda: r.integers(-2**62, 2**62, 16)[x % 16],
+            "kinds": lambda: r.integers(-2**62, 2**62, 1000)[x % 1000], "powers": lambda: np.abs(x) >> r.integers(0, 62, n),
+            "outliers": lambda: np.where(r.random(n) < 0.01, x, np.arange(n)), "short": lambda: x % 40_000}[kind]()
+
+
+@pytest.mark.parametrize("descending", [False, True], ids=["ascending", "descending"])
+@pytest.mark.parametrize("dtype", [np.int32, np.int64, np.float32, np.float64], ids=lambda t: t.__name__)
+@pytest.mark.parametrize("kind", ["half", "most", "beside", "ends", "zipf", "hundred", "thousand", "words", "kinds",
+                                  "powers", "outliers", "short"])
+def test_segments_that_their_range_separates_badly(evo, kind, dtype, descending):
+    """Frequent values among others, values that repeat, magnitudes and outliers:
+    the ways that take over where bins and cuts do not separate the keys, at the
+    sizes where they change, in both directions (floats are cut by value)."""
+    lengths = np.array([40, 300, 512, 513, 1500, 1537, 2048, 2049, 4096, 6144, 8192, 8193, 12_000, 40_003, 300_007])
+    offs = np.concatenate([[0], np.cumsum(lengths)]).astype(np.uint64)
+    r = np.random.default_rng(17)
+    x = uneven(kind, int(offs[-1]), r)
+    if dtype in (np.float32, np.float64):
+        x = x / 2**20
+    elif dtype == np.int32 and np.abs(x).max() >= 2**31:
+        x = x >> 31
+    x = x.astype(dtype)
+    want = oracle.segmented_sort(x, offs)
+    k = torch.from_numpy(x.copy()).cuda()
+    evo.segmented_sort(k, torch.from_numpy(offs.astype(np.int64)).cuda(), descending=descending)
+    evo.sync()
+    if descending:
+        want = np.concatenate([want[int(a):int(b)][::-1] for a, b in zip(offs[:-1], offs[1:])])
+    assert np.array_equal(bits(k), bits(want))
