@@ -633,7 +633,13 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
     // 300 pairs: 5.0 us by passes, 16.7 by insertion; 8,192 pairs of floats with
     // 20 equal ones at most: 36 and 16.5).
     const bool few = IDX && width < 65536ull, strict = !OWN || few || (IDX && n <= 4096);
-    const bool heavy = __syncthreads_or(strict ? (any & (few ? 0xF8F8F8F8u : 0xF0F0F0F0u)) != 0u : widest > 63u);
+    // Up to 1,024 keys a thread that sorts a word of many is what the others wait
+    // for, and the other way is short: words of up to 24 there, of up to 12 in up to
+    // 128 keys, unless a bin is one value and nothing is left to sort (50 floats of
+    // every magnitude: 27.8 us with up to 63, 5.9 so).
+    const bool one_value = !IDX && P::linear && width < (unsigned long long)(4 * WPT * NT);
+    const uint32_t most = !OWN || NT > 512 || n > 1024 || one_value ? 63u : (n > 128 ? 24u : 12u);
+    const bool heavy = __syncthreads_or(strict ? (any & (few ? 0xF8F8F8F8u : 0xF0F0F0F0u)) != 0u : widest > most);
     uint32_t run = inc - sum;
     {
         const uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
@@ -689,7 +695,7 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
     }
     placed();
     __syncthreads();
-    if (!IDX && P::linear && width < (unsigned long long)(4 * WPT * NT)) return k0;   // a bin holds one value
+    if (one_value) return k0;
 
     // ---- words with several keys in a bin: first the pairs, which are most of
     // them, so that a warp's lanes stay together; then the longer ones

@@ -94,8 +94,9 @@ __global__ void __launch_bounds__(NT) small_sort_kernel(const U* in, U* out, con
     bool by_position = true;
     if (ks == nullptr) {
         // frequent values, or keys crowded into a small part of their range:
-        // radix passes over the range, or the merge rounds where they are fewer
-        // (a pass takes about as long as a round: 1.2 us at 1,000 keys)
+        // radix passes over the range, or where they are many, for pairs the
+        // merge rounds if they are fewer (a pass takes about as long as a round:
+        // 1.2 us at 1,000 keys), for keys alone bitonic runs and their merge rounds
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < KPT; ++i)
@@ -108,7 +109,8 @@ __global__ void __launch_bounds__(NT) small_sort_kernel(const U* in, U* out, con
         // shows whether the keys are in order (16 values, 3,000 int64 keys:
         // 27 us by eight passes, 11 so).
         bool lead = false, sorted = false;
-        if (passes > 3) {
+        const bool runs = !PAIRS && NT == kSmallThreads && (n <= 512 || passes > 4 || (passes > 3 && n <= 4096));
+        if (passes > 3 && !(runs && n <= 512)) {
             bool other = false;
             const uint32_t m = __ballot_sync(0xffffffffu, tid < n);
             if (tid < n) {
@@ -143,14 +145,17 @@ __global__ void __launch_bounds__(NT) small_sort_kernel(const U* in, U* out, con
                 quiet = still;
             }
         }
-        if (!sorted) {   // (equal keys are still in input order)
+        ks = nullptr;
+        if constexpr (!PAIRS && NT == kSmallThreads)
+            if (runs && !sorted) ks = smem_sort_any(k0, k1, n);
+        if (!sorted && ks == nullptr) {   // (equal keys are still in input order)
             int rounds = 1;
             while ((kSmallRun << rounds) < n) ++rounds;
             which = passes <= rounds
                         ? smem_radix_sort<U, PAIRS, NT, KPT>(k0, k1, v0, v1, n, lo, 0, passes, counts, sh.wsum)
                         : smem_merge_sort<U, PAIRS, kSmallRun>(k0, k1, v0, v1, n, tins);
         }
-        ks = which ? k1 : k0;
+        if (ks == nullptr) ks = which ? k1 : k0;
         vs = which ? v1 : v0;
         by_position = false;
     }

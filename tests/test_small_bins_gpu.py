@@ -123,3 +123,24 @@ def test_arrays_the_dispatcher_gives_to_one_cta(evo, dtype, kind):
         want = oracle.radix_sort(a)
         assert np.array_equal(bits(y), bits(want)) and np.array_equal(bits(d), bits(want)[::-1]), n
         assert (kinds == ["small"]) == (n <= (15360 if a.itemsize == 4 else 8192)), n
+
+
+def uneven(kind, n, r):
+    x = r.integers(-2**62, 2**62, n)
+    return {"powers": lambda: np.abs(x) >> r.integers(0, 62, n), "zipf": lambda: np.minimum(r.random(n) ** -2.0, 1e6).astype(np.int64),
+            "half": lambda: np.where(r.random(n) < 0.5, 0, x >> 31), "clumps": lambda: (x >> 50 << 50) + r.integers(0, 9, n),
+            "outliers": lambda: np.where(r.random(n) < 0.02, x, np.arange(n) // 3)}[kind]()
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.int64, np.float32, np.float64], ids=lambda t: t.__name__)
+@pytest.mark.parametrize("kind", ["powers", "zipf", "half", "clumps", "outliers"])
+def test_keys_that_crowd_together(evo, kind, dtype):
+    """Words of many keys, which the size limits, and the bitonic runs and merge
+    rounds behind them, at the sizes where they change."""
+    for n in (3, 12, 13, 50, 128, 129, 300, 512, 513, 1024, 1025, 2048, 2049, 3000, 4096, 4097, 8192):
+        x = uneven(kind, n, np.random.default_rng(n))
+        if dtype in (np.float32, np.float64):
+            x = x / 2**20
+        elif dtype == np.int32 and np.abs(x).max() >= 2**31:
+            x = x >> 31
+        check(evo, x.astype(dtype))
