@@ -19,7 +19,7 @@
 // 7.3 ms with 10,240 32-bit counters.
 //
 // Where the stretches do not separate the keys (a bin of 16 keys or more),
-// the caller's own way (OWN) or block_bin_sort_wide takes over: 32-bit counters,
+// the caller's own way (OWN) or block_bin_sort_wide takes over: 16-bit counters,
 // bins of equal keys left as they are, others of up to 32 * kBinWarpKeys keys
 // sorted by one warp each (bitonic), and if some bin is longer still, or the
 // keys crowd together from the start, bitonic runs and the merge rounds of
@@ -350,17 +350,17 @@ __device__ __forceinline__ bool bin_one_value(U* k, int m, BinShared<U, NT>& sh)
 // bin in run, multi: its bins of two or more keys): sorts the bins, the long
 // ones (heavy: there are some) by a warp each, or everything if some bin is
 // longer still and holds several frequent values.
-template <typename U, int NT, int BPT>
+template <typename U, int NT, int WPT>
 __device__ __forceinline__ const U* bin_finish(U* k0, U* k1, int n, uint32_t multi, uint32_t run, bool heavy,
                                                BinShared<U, NT>& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t* const own = (const uint32_t*)k1 + tid * BPT;
+    const uint16_t* const own = (const uint16_t*)k1 + tid * 2 * WPT;
     if (tid == 0) sh.nlist = 0u;
     __syncthreads();
     while (multi) {
         const int q = __ffs((int)multi) - 1;
         multi &= multi - 1u;
-        const uint32_t at = own[q], next = q + 1 < BPT ? own[q + 1] : run;
+        const uint32_t at = own[q], next = q + 1 < 2 * WPT ? own[q + 1] : run;
         const int m = (int)(next - at);
         if (m <= kBinThreadKeys)
             bin_insertion(k0 + at, m);
@@ -435,9 +435,9 @@ struct WidePosition<KeyPosition<U>> {
     }
 };
 
-// The same sort with 32-bit counters and any distribution of the keys, which
-// lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per
-// thread: the words of block_bin_sort, so that k1 is as large as there.  With
+// The same sort with 16-bit counters, two to a word, and any distribution of the
+// keys, which lie in k0 (element i * NT + thread of a thread, n in all).  WPT
+// words per thread as in block_bin_sort, so that k1 is as large as there.  With
 // ask, one key of each thread tells first whether bins can separate them at all
 // (a quarter of these keys share a 1024th of the range with a different one: they
 // cannot), and whether some value is so frequent that a warp's equal bins are
@@ -445,13 +445,15 @@ struct WidePosition<KeyPosition<U>> {
 // 2,000 segments of 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose
 // values crowd together are tried once more by their bit patterns, which spread
 // magnitudes evenly.  Bins of one value are left as they are: 1e8 int64 keys with
-// some 40 keys of each value, partition sort, 23.2 -> 3.7 ms (every bin by a warp
-// before, or everything merged).
-template <typename U, int NT, int KPT, int BPT, typename P>
+// some 40 keys of each value, partition sort, 23.2 -> 3.5 ms (every bin by a warp
+// before, or everything merged); with some 10, 3.06 -> 2.87 ms against 32-bit
+// counters, half as many bins.
+template <typename U, int NT, int KPT, int WPT, typename P>
 __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, WidePosition<P> given,
                                                      bool ask, U* k0, U* k1, BinShared<U, NT>& sh) {
     const P position = given.get(lo, width);
-    static_assert(BPT % 8 == 4 && BPT * NT <= kBinMax, "bins per thread");
+    static_assert(WPT % 8 == 4 && 2 * WPT <= 32 && 2 * WPT * NT <= kBinMax, "words per thread");
+    constexpr uint32_t BINS = 2 * WPT * NT;
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool add_up = false;
@@ -463,22 +465,22 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
             if constexpr (P::linear)
                 return smem_sort_any(k0, k1, n);
             else
-                return block_bin_sort_wide<U, NT, KPT, BPT, KeyPosition<U>>(
+                return block_bin_sort_wide<U, NT, KPT, WPT, KeyPosition<U>>(
                     n, lo, width, WidePosition<KeyPosition<U>>(), true, k0, k1, sh);
         }
         add_up = 4 * __syncthreads_count(v.frequent) > most;
     }
-    uint32_t* const bins = (uint32_t*)k1;
-    // A thread's BPT bins are consecutive and read four at a time; with BPT / 4
+    uint32_t* const words = (uint32_t*)k1;
+    // A thread's WPT words are consecutive and read four at a time; with WPT / 4
     // odd, a quarter-warp's 16-byte reads fall in different banks.
-    uint4* const mine = (uint4*)bins + tid * (BPT / 4);
-    bin_zero<NT, BPT>(k1);
+    uint4* const mine = (uint4*)words + tid * (WPT / 4);
+    bin_zero<NT, WPT>(k1);
     U key[KPT];
 #pragma unroll
     for (int i = 0; i < KPT; ++i) key[i] = i * NT + tid < n ? k0[i * NT + tid] : (U)0;
     int lz;
-    uint32_t mult = (uint32_t)(BPT * NT);
-    if (P::linear) cut_range(width, (uint32_t)(BPT * NT), &lz, &mult);
+    uint32_t mult = BINS;
+    if (P::linear) cut_range(width, BINS, &lz, &mult);
     const uint32_t lt = lanemask_lt();
     __syncthreads();
     // ---- count; the old count is the key's place in its bin
@@ -489,16 +491,16 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         const uint32_t some = __ballot_sync(0xffffffffu, have);
         if (have) {
             // (in range for every key of [lo, lo + width]; never out of the array for any other)
-            const uint32_t b = min(__umulhi(position(key[i]), mult), (uint32_t)(BPT * NT - 1));
+            const uint32_t b = min(__umulhi(position(key[i]), mult), BINS - 1u), half = 16u * (b & 1u);
             uint32_t place;
             if (add_up) {
                 const uint32_t peers = __match_any_sync(some, b);
                 const int leader = __ffs((int)peers) - 1;
                 place = 0u;
-                if (lane == leader) place = atomicAdd(&bins[b], (uint32_t)__popc(peers));
+                if (lane == leader) place = atomicAdd(&words[b >> 1], (uint32_t)__popc(peers) << half) >> half & 0xFFFFu;
                 place = __shfl_sync(peers, place, leader) + (uint32_t)__popc(peers & lt);
             } else {
-                place = atomicAdd(&bins[b], 1u);
+                place = atomicAdd(&words[b >> 1], 1u << half) >> half & 0xFFFFu;
             }
             br[i] = b | place << 16;
         }
@@ -508,14 +510,18 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
     // ---- exclusive scan of the bins
     uint32_t sum = 0, multi = 0, any = 0;   // multi: bins of two or more keys
 #pragma unroll
-    for (int j = 0; j < BPT / 4; ++j) {
+    for (int j = 0; j < WPT / 4; ++j) {
         const uint4 q = mine[j];
-        sum += q.x + q.y + q.z + q.w;
         any |= q.x | q.y | q.z | q.w;
-        if (q.x > 1u) multi |= 1u << (4 * j);
-        if (q.y > 1u) multi |= 2u << (4 * j);
-        if (q.z > 1u) multi |= 4u << (4 * j);
-        if (q.w > 1u) multi |= 8u << (4 * j);
+        auto word = [&](uint32_t x, int at) {
+            sum += (x & 0xFFFFu) + (x >> 16);
+            if (x & 0xFFFEu) multi |= 1u << at;
+            if (x >> 17) multi |= 2u << at;
+        };
+        word(q.x, 8 * j);
+        word(q.y, 8 * j + 2);
+        word(q.z, 8 * j + 4);
+        word(q.w, 8 * j + 6);
     }
     uint32_t inc = sum;
 #pragma unroll
@@ -532,23 +538,30 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         run += __reduce_add_sync(0xffffffffu, v);
     }
 #pragma unroll
-    for (int j = 0; j < BPT / 4; ++j) {
+    for (int j = 0; j < WPT / 4; ++j) {
         uint4 q = mine[j];   // read again: registers hold the keys
-        const uint32_t a = run + q.x, b = a + q.y, c = b + q.z, d = c + q.w;
-        q = make_uint4(run, a, b, c);
+        auto word = [&](uint32_t x) {   // counts -> first places (n < 2^14)
+            const uint32_t v = run | (run + (x & 0xFFFFu)) << 16;
+            run += (x & 0xFFFFu) + (x >> 16);
+            return v;
+        };
+        q.x = word(q.x);
+        q.y = word(q.y);
+        q.z = word(q.z);
+        q.w = word(q.w);
         mine[j] = q;
-        run = d;
     }
-    const bool one_value = P::linear && width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
-    const bool heavy = __syncthreads_or(!one_value && any > (uint32_t)kBinThreadKeys);
+    const bool one_value = P::linear && width < (unsigned long long)BINS;   // per bin: nothing left to sort
+    const bool heavy = __syncthreads_or(!one_value && (any & 0xFFE0FFE0u) != 0u);
+    static_assert(kBinThreadKeys == 31, "the bits above");
 
     // ---- every key to its place
 #pragma unroll
     for (int i = 0; i < KPT; ++i)
-        if (i * NT + tid < n) k0[bins[br[i] & 0xFFFFu] + (br[i] >> 16)] = key[i];
+        if (i * NT + tid < n) k0[((const uint16_t*)k1)[br[i] & 0xFFFFu] + (br[i] >> 16)] = key[i];
     __syncthreads();
     if (one_value) return k0;
-    return bin_finish<U, NT, BPT>(k0, k1, n, multi, run, heavy, sh);
+    return bin_finish<U, NT, WPT>(k0, k1, n, multi, run, heavy, sh);
 }
 
 // Sorts the n keys that the CTA's NT threads hold in registers (key i of a
