@@ -609,15 +609,25 @@ def segmented_block_cap(path, w, total):
 
 
 def segmented_alg_bytes(lens, w, block_cap):
-    """Algorithmic bytes of one batched segmented sort: 2w per key for a
+    """Bytes of one batched segmented sort by digit passes: 2w per key for a
     segment one CTA sorts on chip, and the radix formula w + P * 2w per key
     (P = 8w / 8 passes of 8-bit digits, all active for full-range keys) for
-    the longer ones."""
+    the longer ones (segmented_moved_bytes: what the cut of long segments moves)."""
     import torch
     lens = torch.as_tensor(lens, dtype=torch.int64)
     small = int(lens[lens <= block_cap].sum())
     big = int(lens[lens > block_cap].sum())
     return 2 * w * small + (w + w * 2 * w) * big
+
+
+def segmented_moved_bytes(lens, w, block_cap):
+    """Bytes the segmented sort's kernel moves: 2w per key for a segment one CTA
+    sorts on chip; 5w for a longer one (read to count, read and written to its
+    part, read and written by the sort on chip)."""
+    import torch
+    lens = torch.as_tensor(lens, dtype=torch.int64)
+    small = int(lens[lens <= block_cap].sum())
+    return 2 * w * small + 5 * w * (int(lens.sum()) - small)
 
 
 def leg_segmented(evo, args, stream, barrier, dev, nseg=100_000, rank=0, world=1):
@@ -697,7 +707,7 @@ def leg_segmented(evo, args, stream, barrier, dev, nseg=100_000, rank=0, world=1
     plain_ms = _time_steps(per_array, 1, 1, stream) - copy_ms
     evo.sync()
     cap = segmented_block_cap(os.path.join(TABLE_DIR, "gb300_int32.txt"), 4, total)
-    alg = segmented_alg_bytes(lens, 4, cap)
+    alg = segmented_moved_bytes(lens, 4, cap)
     peak, peak_src = measured_peaks()
     ach = alg / 1e9 / (ms_t * 1e-3)
     seg_roof = {"bound": "hbm", "kernel": "seg_sort (whole batch, one persistent launch)", "achieved": ach,
@@ -772,7 +782,8 @@ def small_graph_us(evo, x, y, kw, reps=100):
 
 def leg_small(evo, args, stream, barrier, dev):
     """Latency of small sorts: the dispatcher's one-CTA path (the default for
-    arrays up to 4096 keys) against the device-wide radix path, per call."""
+    arrays up to 15,360 32-bit keys, 8,192 others) against the device-wide radix
+    path, per call."""
     import torch
     from paper_2505_18681_gb300 import inputs
     # no tuned table: above the one-CTA cut-over 'auto' then takes the default
@@ -810,7 +821,7 @@ def leg_small(evo, args, stream, barrier, dev):
                           "graph_us_per_sort": small_graph_us(evo, x, y, kw)}
         res[str(n)] = row
     return {"unit": "us per sort", "config": {"workload": "one int32 array of 1e3 / 4096 / 1e4 uniform keys per call; "
-                                              "'auto' lets the dispatcher choose (one-CTA path up to 4096 keys), "
+                                              "'auto' lets the dispatcher choose (one-CTA path up to 15,360 32-bit keys), "
                                               "'radix' forces the device-wide radix sort; call_us: events around "
                                               "the Python call on its stream (includes host overhead), "
                                               "kernel_us: the library's events around its launches (includes "

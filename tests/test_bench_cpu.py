@@ -160,3 +160,10 @@ def test_reference_line_carries_the_contract_keys(monkeypatch, capsys):
     e = line["e2e"]
     assert e["value"] == line["value"] and e["unit"] == line["unit"]
     assert e["h2d_bytes_per_step"] == 0 and e["d2h_bytes_per_step"] == 0
+
+
+def test_segmented_roofline_counts_what_the_cut_moves():
+    """A segment past the block cap is read to be counted, moved to its parts and
+    sorted on chip: five key widths, whatever the width."""
+    assert bench.segmented_moved_bytes([10, 100, 5000], 4, 4096) == 2 * 4 * 110 + 5 * 4 * 5000
+    assert bench.segmented_moved_bytes([4096, 4097], 8, 4096) == 2 * 8 * 4096 + 5 * 8 * 4097
