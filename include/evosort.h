@@ -197,15 +197,18 @@ evosort_status evosort_resolve(size_t n, evosort_dtype dt, int with_values, cons
  * keys' span needs fewer 8-bit digits than their raw digits that vary (a
  * decision taken on the device).
  * With 8-bit digits and no tile, ranking or pass kernel asked for, arrays
- * above the one-CTA path and up to 1.3e6 (64-bit pairs) .. 2.5e6 (32-bit
- * keys) elements are radix sorted by one cooperative launch (the chain of
- * launches where the device cannot hold its CTAs at once); AUTO sorts of
- * fewer than 2^16 elements that it takes read no sample unless the table names
- * the mergesort for the key type.  Larger AUTO sorts of keys alone try two
- * partition steps and sorts in shared memory first (keys of at least 2^21
- * elements with a table, which read one more small result back, of 2^23
- * without, which stay asynchronous), in the same scratch memory, and fall
- * back to the radix passes where the keys do not spread.  Whatever the path,
+ * above the one-CTA path and up to 1,024 per SM times 16 (32-bit keys), 12
+ * (64-bit keys, or 32-bit keys with values) or 8 (64-bit keys with values)
+ * elements, 2.49e6, 1.87e6 and 1.25e6 on 152 SMs, are radix sorted by one
+ * cooperative launch (the chain of launches where the device cannot hold its
+ * CTAs at once); AUTO sorts of fewer than 2^16 elements that it takes read no
+ * sample unless the table names the mergesort for the key type; the tile of a
+ * table's entry is for the chain of launches, which larger sorts take.  Larger
+ * AUTO sorts of keys alone try two partition steps and sorts in shared memory
+ * first (keys of at least 2^21 elements with a table, which read one more small
+ * result back, of 2^23 without, which stay asynchronous; of 2^26 where the keys
+ * span 24 bits or less), in the same scratch memory, and fall back to the radix
+ * passes where the keys do not spread.  Whatever the path,
  * the result is the one sorted array. */
 evosort_status evosort_sort(void* keys, size_t n, evosort_dtype dt, const evosort_params* p);
 

@@ -208,8 +208,11 @@ cudaError_t launch_small(const void* in, void* out, const uint32_t* vin, uint32_
 // Against the one-launch radix sort, whose barriers over the grid take it 37 us
 // for 32-bit and 57 to 64 us for 64-bit keys at these sizes: 10,000 uniform
 // int32 keys 9.5 us, 15,360 12.0, 8,192 uniform int64 keys 11.4, with values
-// 15.5.  Keys that the bins do not separate are about even (Zipf, 8,192 int32 keys
-// 26.6 and 26.8 us, 15,360 42 and 31).
+// 15.5.  Keys that the bins do not separate lose to it from some 8,000 on, whatever
+// repeats or crowds together in them (int32, one CTA and one launch, us): 8,192 keys
+// Zipf 29 and 27, exponential 46 and 33; 12,000 of a thousand small values 27 and 15;
+// 15,360 Zipf 46 and 31, half of them equal 54 and 38, magnitudes of every order 56
+// and 37.  (The chain of launches that such sorts took before: 75 to 90.)
 size_t small_auto_keys(int w, bool pairs) {
     return w == 4 && !pairs ? (size_t)kSmallWideKpt * kSmallWideThreads : (size_t)kSmallMax;
 }

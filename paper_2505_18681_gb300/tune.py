@@ -112,7 +112,8 @@ def tune_table(dtype=torch.int64, n=1 << 28, classes=None, seed=42, population=3
 def tune_segmented(dtype=torch.int32, nseg=10_000, lo=16, hi=1_000_000, seed=42, population=30, generations=10,
                    reps=3, verbose=True):
     """GA over the segmented sort's tier cut-overs (warp tier, block tier,
-    giant segments) and the block tier's insertion threshold, on a batch of
+    giant segments; the insertion threshold is still drawn and recorded, but
+    no tier has insertion-sorted runs any more), on a batch of
     nseg segments with log-uniform lengths lo..hi (half uniform, half nearly
     sorted keys).  Fitness: the median device time of the batched sort; a
     candidate whose output differs from the reference batch sort (made once
