@@ -19,11 +19,11 @@
 // 7.3 ms with 10,240 32-bit counters.
 //
 // Where the stretches do not separate the keys (a bin of 16 keys or more),
-// the caller's own way (OWN) or block_bin_sort_wide takes over: 16-bit counters,
-// bins of equal keys left as they are, others of up to 32 * kBinWarpKeys keys
-// sorted by one warp each (bitonic), and if some bin is longer still, or the
-// keys crowd together from the start, bitonic runs and the merge rounds of
-// Algorithm 3, so any input is sorted in bounded time.
+// the caller's own way (OWN) or block_bin_sort_fine or _wide takes over: counters
+// of 16 or 32 bits, bins of equal keys left as they are, others of up to 32 *
+// kBinWarpKeys keys sorted by one warp each (bitonic), and if some bin is longer
+// still, or the keys crowd together from the start, bitonic runs and the merge
+// rounds of Algorithm 3, so any input is sorted in bounded time.
 #pragma once
 
 #include <cfloat>
@@ -346,45 +346,66 @@ __device__ __forceinline__ bool bin_one_value(U* k, int m, BinShared<U, NT>& sh)
     return true;
 }
 
-// The keys of k0 stand in their bins (starts in k1, ends of a thread's last
-// bin in run, multi: its bins of two or more keys): sorts the bins, the long
-// ones (heavy: there are some) by a warp each, or everything if some bin is
-// longer still and holds several frequent values.
-template <typename U, int NT, int WPT>
-__device__ __forceinline__ const U* bin_finish(U* k0, U* k1, int n, uint32_t multi, uint32_t run, bool heavy,
-                                               BinShared<U, NT>& sh) {
+// The keys of k0 stand in their bins (starts in k1, of type C, ends of a thread's
+// last bin in run, multi: its bins of two or more keys): sorts the bins.  A thread
+// sorts its short ones, up to kBinThreadWork steps or so in all: where keys crowd
+// together the bins of one thread may hold hundreds.  The others are sorted by a
+// warp each, or everything if some bin is very long and holds several frequent
+// values.
+constexpr int kBinThreadWork = 256;
+template <typename U, int NT, int BPT, typename C>
+__device__ __forceinline__ const U* bin_finish(U* k0, U* k1, int n, uint32_t multi, uint32_t run, BinShared<U, NT>& sh) {
+    constexpr int ROOM = sizeof(sh.list) / sizeof(sh.list[0]);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint16_t* const own = (const uint16_t*)k1 + tid * 2 * WPT;
-    if (tid == 0) sh.nlist = 0u;
+    const C* const own = (const C*)k1 + tid * BPT;
+    if (tid == 0) sh.nlist = sh.nodd = 0u;
     __syncthreads();
+    int work = 0;
     while (multi) {
         const int q = __ffs((int)multi) - 1;
         multi &= multi - 1u;
-        const uint32_t at = own[q], next = q + 1 < 2 * WPT ? own[q + 1] : run;
+        const uint32_t at = own[q], next = q + 1 < BPT ? own[q + 1] : run;
         const int m = (int)(next - at);
-        if (m <= kBinThreadKeys)
-            bin_insertion(k0 + at, m);
-        else
-            sh.list[atomicAdd(&sh.nlist, 1u)] = at | (uint32_t)m << 16;   // n / (kBinThreadKeys + 1) entries at most
+        work += m * m / 4;
+        // (bins of more than kBinThreadKeys: n / (kBinThreadKeys + 1) at most, which is half the room)
+        bool mine = m <= kBinThreadKeys && (work <= kBinThreadWork || m <= 4);
+        if (!mine) {
+            const uint32_t e = atomicAdd(m <= kBinThreadKeys ? &sh.nodd : &sh.nlist, 1u);
+            if (m > kBinThreadKeys)
+                sh.list[e] = at | (uint32_t)m << 16;
+            else if (e < ROOM / 2)
+                sh.list[ROOM - 1 - e] = at | (uint32_t)m << 16;
+            else
+                mine = true;
+        }
+        if (mine) bin_insertion(k0 + at, m);
     }
     __syncthreads();
-    if (!heavy) return k0;
-    const int listed = (int)sh.nlist;
+    const int listed = (int)sh.nlist, shorter = min((int)sh.nodd, ROOM / 2);
+    __syncthreads();   // (nodd is used again)
     for (int e = 0; e < listed; ++e) {
         const int m = (int)(sh.list[e] >> 16);
         if (m > 32 * kBinWarpKeys && !bin_one_value<U, NT>(k0 + (sh.list[e] & 0xFFFFu), m, sh))
             return smem_sort_any(k0, k1, n);   // (k1's starts are not needed any more)
     }
-    for (int e = warp; e < listed; e += NT / 32) {
-        U* const k = k0 + (sh.list[e] & 0xFFFFu);
-        const int m = (int)(sh.list[e] >> 16);
+    for (int e = warp; e < listed + shorter; e += NT / 32) {
+        const uint32_t x = e < listed ? sh.list[e] : sh.list[ROOM - 1 - (e - listed)];
+        U* const k = k0 + (x & 0xFFFFu);
+        const int m = (int)(x >> 16);
         if (m > 32 * kBinWarpKeys) continue;
+        if (m <= 32) {
+            U one[1] = {lane < m ? k[lane] : ~(U)0};
+            __syncwarp();
+            warp_bitonic_sort<U, 1>(one);
+            if (lane < m) k[lane] = one[0];
+            continue;
+        }
         const U first = k[0];
         bool other = false;
         for (int i = lane; i < m; i += 32) other |= k[i] != first;
         if (__any_sync(0xffffffffu, other)) bin_warp_sort(k, m);
     }
-    __syncthreads();
+    if (listed + shorter) __syncthreads();
     return k0;
 }
 
@@ -435,29 +456,28 @@ struct WidePosition<KeyPosition<U>> {
     }
 };
 
-// The same sort with 16-bit counters, two to a word, and any distribution of the
-// keys, which lie in k0 (element i * NT + thread of a thread, n in all).  WPT
-// words per thread as in block_bin_sort, so that k1 is as large as there.  With
-// ask, one key of each thread tells first whether bins can separate them at all
-// (a quarter of these keys share a 1024th of the range with a different one: they
-// cannot), and whether some value is so frequent that a warp's equal bins are
-// better added up before the counters see them (it costs more where they differ:
-// 2,000 segments of 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose
-// values crowd together are tried once more by their bit patterns, which spread
-// magnitudes evenly.  Bins of one value are left as they are: 1e8 int64 keys with
-// some 40 keys of each value, partition sort, 23.2 -> 3.5 ms (every bin by a warp
-// before, or everything merged); with some 10, 3.06 -> 2.87 ms against 32-bit
-// counters, half as many bins.
-template <typename U, int NT, int KPT, int WPT, typename P>
+// The same sort with 32-bit counters and any distribution of the keys, which
+// lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per
+// thread: the words of block_bin_sort, so that k1 is as large as there.  One key
+// of each thread tells first whether bins can separate them at all (a quarter of
+// these keys share a 1024th of the range with a different one: they cannot), and
+// whether some value is so frequent that a warp's equal bins are better added up
+// before the counters see them (it costs more where they differ: 2,000 segments of
+// 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose values crowd together
+// are tried once more by their bit patterns, which spread magnitudes evenly.
+// Bins of one value are left as they are: 1e8 int64 keys with some 40 keys of each
+// value, partition sort, 23.2 -> 3.7 ms (every bin by a warp before, or everything
+// merged).
+template <typename U, int NT, int KPT, int BPT, typename P>
 __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, WidePosition<P> given,
-                                                     bool ask, U* k0, U* k1, BinShared<U, NT>& sh) {
+                                                     U* k0, U* k1, BinShared<U, NT>& sh) {
     const P position = given.get(lo, width);
-    static_assert(WPT % 8 == 4 && 2 * WPT <= 32 && 2 * WPT * NT <= kBinMax, "words per thread");
-    constexpr uint32_t BINS = 2 * WPT * NT;
+    static_assert(BPT % 8 == 4 && BPT * NT <= kBinMax, "bins per thread");
+    static_assert(KPT * NT <= 256 * (kBinThreadKeys + 1), "half of the list");
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    bool add_up = false;
-    if (ask) {
+    bool add_up;
+    {
         const int at = lane % ((n + NT - 1) / NT) * NT + tid;
         const KeyVotes v = key_votes(at < n ? k0[at] : (U)0, at < n, position);
         const int most = min(n, NT);
@@ -465,11 +485,107 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
             if constexpr (P::linear)
                 return smem_sort_any(k0, k1, n);
             else
-                return block_bin_sort_wide<U, NT, KPT, WPT, KeyPosition<U>>(
-                    n, lo, width, WidePosition<KeyPosition<U>>(), true, k0, k1, sh);
+                return block_bin_sort_wide<U, NT, KPT, BPT, KeyPosition<U>>(
+                    n, lo, width, WidePosition<KeyPosition<U>>(), k0, k1, sh);
         }
         add_up = 4 * __syncthreads_count(v.frequent) > most;
     }
+    uint32_t* const bins = (uint32_t*)k1;
+    // A thread's BPT bins are consecutive and read four at a time; with BPT / 4
+    // odd, a quarter-warp's 16-byte reads fall in different banks.
+    uint4* const mine = (uint4*)bins + tid * (BPT / 4);
+    bin_zero<NT, BPT>(k1);
+    U key[KPT];
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) key[i] = i * NT + tid < n ? k0[i * NT + tid] : (U)0;
+    int lz;
+    uint32_t mult = (uint32_t)(BPT * NT);
+    if (P::linear) cut_range(width, (uint32_t)(BPT * NT), &lz, &mult);
+    const uint32_t lt = lanemask_lt();
+    __syncthreads();
+    // ---- count; the old count is the key's place in its bin
+    uint32_t br[KPT];   // bin | place << 16
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        const bool have = i * NT + tid < n;
+        const uint32_t some = __ballot_sync(0xffffffffu, have);
+        if (have) {
+            // (in range for every key of [lo, lo + width]; never out of the array for any other)
+            const uint32_t b = min(__umulhi(position(key[i]), mult), (uint32_t)(BPT * NT - 1));
+            uint32_t place;
+            if (add_up) {
+                const uint32_t peers = __match_any_sync(some, b);
+                const int leader = __ffs((int)peers) - 1;
+                place = 0u;
+                if (lane == leader) place = atomicAdd(&bins[b], (uint32_t)__popc(peers));
+                place = __shfl_sync(peers, place, leader) + (uint32_t)__popc(peers & lt);
+            } else {
+                place = atomicAdd(&bins[b], 1u);
+            }
+            br[i] = b | place << 16;
+        }
+    }
+    __syncthreads();
+
+    // ---- exclusive scan of the bins
+    uint32_t sum = 0, multi = 0;   // multi: bins of two or more keys
+#pragma unroll
+    for (int j = 0; j < BPT / 4; ++j) {
+        const uint4 q = mine[j];
+        sum += q.x + q.y + q.z + q.w;
+        if (q.x > 1u) multi |= 1u << (4 * j);
+        if (q.y > 1u) multi |= 2u << (4 * j);
+        if (q.z > 1u) multi |= 4u << (4 * j);
+        if (q.w > 1u) multi |= 8u << (4 * j);
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sh.wsum[warp] = inc;
+    __syncthreads();
+    uint32_t run = inc - sum;
+    {
+        uint32_t v = lane < NW ? sh.wsum[lane] : 0u;
+        v = lane < warp ? v : 0u;
+        run += __reduce_add_sync(0xffffffffu, v);
+    }
+#pragma unroll
+    for (int j = 0; j < BPT / 4; ++j) {
+        uint4 q = mine[j];   // read again: registers hold the keys
+        const uint32_t a = run + q.x, b = a + q.y, c = b + q.z, d = c + q.w;
+        q = make_uint4(run, a, b, c);
+        mine[j] = q;
+        run = d;
+    }
+    const bool one_value = P::linear && width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
+    __syncthreads();
+
+    // ---- every key to its place
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+        if (i * NT + tid < n) k0[bins[br[i] & 0xFFFFu] + (br[i] >> 16)] = key[i];
+    __syncthreads();
+    if (one_value) return k0;
+    return bin_finish<U, NT, BPT, uint32_t>(k0, k1, n, multi, run, sh);
+}
+
+// The same for keys of which no bin of block_bin_sort held 32: two 16-bit counters
+// to a word, so that fewer values share a bin.  (Not for frequent keys: the shared
+// atomic that adds one constant counts equal ones of a warp at once, this one
+// does not.)  1e8 keys with some ten copies of each value: int32 2.21 -> 2.07 ms,
+// int64 3.06 -> 2.87 ms.
+template <typename U, int NT, int KPT, int WPT, typename P>
+__device__ __noinline__ const U* block_bin_sort_fine(int n, U lo, unsigned long long width, WidePosition<P> given,
+                                                     U* k0, U* k1, BinShared<U, NT>& sh) {
+    const P position = given.get(lo, width);
+    static_assert(WPT % 8 == 4 && 2 * WPT <= 32 && 2 * WPT * NT <= kBinMax, "words per thread");
+    static_assert(KPT * NT <= 256 * (kBinThreadKeys + 1), "half of the list");
+    constexpr uint32_t BINS = 2 * WPT * NT;
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t* const words = (uint32_t*)k1;
     // A thread's WPT words are consecutive and read four at a time; with WPT / 4
     // odd, a quarter-warp's 16-byte reads fall in different banks.
@@ -481,38 +597,24 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
     int lz;
     uint32_t mult = BINS;
     if (P::linear) cut_range(width, BINS, &lz, &mult);
-    const uint32_t lt = lanemask_lt();
     __syncthreads();
     // ---- count; the old count is the key's place in its bin
     uint32_t br[KPT];   // bin | place << 16
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-        const bool have = i * NT + tid < n;
-        const uint32_t some = __ballot_sync(0xffffffffu, have);
-        if (have) {
+        if (i * NT + tid < n) {
             // (in range for every key of [lo, lo + width]; never out of the array for any other)
             const uint32_t b = min(__umulhi(position(key[i]), mult), BINS - 1u), half = 16u * (b & 1u);
-            uint32_t place;
-            if (add_up) {
-                const uint32_t peers = __match_any_sync(some, b);
-                const int leader = __ffs((int)peers) - 1;
-                place = 0u;
-                if (lane == leader) place = atomicAdd(&words[b >> 1], (uint32_t)__popc(peers) << half) >> half & 0xFFFFu;
-                place = __shfl_sync(peers, place, leader) + (uint32_t)__popc(peers & lt);
-            } else {
-                place = atomicAdd(&words[b >> 1], 1u << half) >> half & 0xFFFFu;
-            }
-            br[i] = b | place << 16;
+            br[i] = b | (atomicAdd(&words[b >> 1], 1u << half) >> half & 0xFFFFu) << 16;
         }
     }
     __syncthreads();
 
     // ---- exclusive scan of the bins
-    uint32_t sum = 0, multi = 0, any = 0;   // multi: bins of two or more keys
+    uint32_t sum = 0, multi = 0;   // multi: bins of two or more keys
 #pragma unroll
     for (int j = 0; j < WPT / 4; ++j) {
         const uint4 q = mine[j];
-        any |= q.x | q.y | q.z | q.w;
         auto word = [&](uint32_t x, int at) {
             sum += (x & 0xFFFFu) + (x >> 16);
             if (x & 0xFFFEu) multi |= 1u << at;
@@ -552,8 +654,7 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         mine[j] = q;
     }
     const bool one_value = P::linear && width < (unsigned long long)BINS;   // per bin: nothing left to sort
-    const bool heavy = __syncthreads_or(!one_value && (any & 0xFFE0FFE0u) != 0u);
-    static_assert(kBinThreadKeys == 31, "the bits above");
+    __syncthreads();
 
     // ---- every key to its place
 #pragma unroll
@@ -561,7 +662,7 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         if (i * NT + tid < n) k0[((const uint16_t*)k1)[br[i] & 0xFFFFu] + (br[i] >> 16)] = key[i];
     __syncthreads();
     if (one_value) return k0;
-    return bin_finish<U, NT, WPT>(k0, k1, n, multi, run, heavy, sh);
+    return bin_finish<U, NT, 2 * WPT, uint16_t>(k0, k1, n, multi, run, sh);
 }
 
 // Sorts the n keys that the CTA's NT threads hold in registers (key i of a
@@ -666,8 +767,9 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
                     if (i * NT + tid < n) k0[i * NT + tid] = key[i];
                 // (bins of fewer than 32 keys: the threads sort them, whatever the keys)
                 const bool mild = !__syncthreads_or((any & 0xE0E0E0E0u) != 0u) && __reduce_add_sync(0xffffffffu, v) == (uint32_t)n;
-                const U* r = block_bin_sort_wide<U, NT, KPT, WPT, P>(n, lo, width, WidePosition<P>(position), !mild, k0,
-                                                                     k1, sh);
+                const WidePosition<P> given(position);
+                const U* r = mild ? block_bin_sort_fine<U, NT, KPT, WPT, P>(n, lo, width, given, k0, k1, sh)
+                                  : block_bin_sort_wide<U, NT, KPT, WPT, P>(n, lo, width, given, k0, k1, sh);
                 placed();
                 return r;
             }
