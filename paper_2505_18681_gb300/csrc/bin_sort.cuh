@@ -458,16 +458,16 @@ struct WidePosition<KeyPosition<U>> {
 
 // The same sort with 32-bit counters and any distribution of the keys, which
 // lie in k0 (element i * NT + thread of a thread, n in all).  BPT bins per
-// thread: the words of block_bin_sort, so that k1 is as large as there.  One key
-// of each thread tells first whether bins can separate them at all (a quarter of
-// these keys share a 1024th of the range with a different one: they cannot), and
-// whether some value is so frequent that a warp's equal bins are better added up
-// before the counters see them (it costs more where they differ: 2,000 segments of
-// 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose values crowd together
-// are tried once more by their bit patterns, which spread magnitudes evenly.
-// Bins of one value are left as they are: 1e8 int64 keys with some 40 keys of each
-// value, partition sort, 23.2 -> 3.7 ms (every bin by a warp before, or everything
-// merged).
+// thread: the words of block_bin_sort, so that k1 is as large as there.  Unless a
+// bin is one value, one key of each thread tells first whether bins can separate
+// them at all (a quarter of these keys share a 1024th of the range with a different
+// one: they cannot), and whether some value is so frequent that a warp's equal bins
+// are better added up before the counters see them (it costs more where they
+// differ: 2,000 segments of 4,000 int32 keys of 7 values 95 -> 109 us).  Floats whose
+// values crowd together are tried once more by their bit patterns, which spread
+// magnitudes evenly.  Bins of one value are left as they are: 1e8 int64 keys with
+// some 40 keys of each value, partition sort, 23.2 -> 3.6 ms (every bin by a warp
+// before, or everything merged).
 template <typename U, int NT, int KPT, int BPT, typename P>
 __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long long width, WidePosition<P> given,
                                                      U* k0, U* k1, BinShared<U, NT>& sh) {
@@ -476,8 +476,9 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
     static_assert(KPT * NT <= 256 * (kBinThreadKeys + 1), "half of the list");
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    bool add_up;
-    {
+    const bool one_value = P::linear && width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
+    bool add_up = false;
+    if (!one_value) {
         const int at = lane % ((n + NT - 1) / NT) * NT + tid;
         const KeyVotes v = key_votes(at < n ? k0[at] : (U)0, at < n, position);
         const int most = min(n, NT);
@@ -560,7 +561,6 @@ __device__ __noinline__ const U* block_bin_sort_wide(int n, U lo, unsigned long 
         mine[j] = q;
         run = d;
     }
-    const bool one_value = P::linear && width < (unsigned long long)(BPT * NT);   // per bin: nothing left to sort
     __syncthreads();
 
     // ---- every key to its place
@@ -765,8 +765,10 @@ __device__ __forceinline__ const U* block_bin_sort(const U (&key)[KPT], int n, U
 #pragma unroll
                 for (int i = 0; i < KPT; ++i)
                     if (i * NT + tid < n) k0[i * NT + tid] = key[i];
-                // (bins of fewer than 32 keys: the threads sort them, whatever the keys)
-                const bool mild = !__syncthreads_or((any & 0xE0E0E0E0u) != 0u) && __reduce_add_sync(0xffffffffu, v) == (uint32_t)n;
+                // (bins of fewer than 32 keys; one value each needs no sort at all)
+                const bool single = P::linear && width < (unsigned long long)(WPT * NT);
+                const bool mild = !single && !__syncthreads_or((any & 0xE0E0E0E0u) != 0u) &&
+                                  __reduce_add_sync(0xffffffffu, v) == (uint32_t)n;
                 const WidePosition<P> given(position);
                 const U* r = mild ? block_bin_sort_fine<U, NT, KPT, WPT, P>(n, lo, width, given, k0, k1, sh)
                                   : block_bin_sort_wide<U, NT, KPT, WPT, P>(n, lo, width, given, k0, k1, sh);

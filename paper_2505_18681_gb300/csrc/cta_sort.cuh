@@ -375,7 +375,7 @@ __device__ __forceinline__ bool cta_split_impl(U* src, U* part, U* fin, uint32_t
     // ---- range of the keys, from a sample, and whether to cut them at all
     U lo, hi;
     float low = 0.f, scale = 0.f;   // floats: the cut of the sampled values
-    bool passes;
+    bool passes = false;   // (asked of whole runs only)
     {
         U k[8];
         const uint32_t stride = len / (8 * kCtaThreads);
@@ -389,9 +389,10 @@ __device__ __forceinline__ bool cta_split_impl(U* src, U* part, U* fin, uint32_t
             const auto pos = block_value_position<U, kCtaThreads, 8>(k, m, out, out.descending(), sh.value);
             low = pos.low;
             scale = pos.scale;
-            passes = cta_wants_passes<U>(k, m, len, lo, 0ull, pos, sh);
+            if (LEVEL == 0) passes = cta_wants_passes<U>(k, m, len, lo, 0ull, pos, sh);
         } else {
-            passes = cta_wants_passes<U>(k, m, len, lo, (unsigned long long)(U)(hi - lo), KeyPosition<U>{lo, wlz}, sh);
+            if (LEVEL == 0)
+                passes = cta_wants_passes<U>(k, m, len, lo, (unsigned long long)(U)(hi - lo), KeyPosition<U>{lo, wlz}, sh);
         }
     }
     const unsigned long long width = (unsigned long long)(U)(hi - lo);
